@@ -121,7 +121,7 @@ struct CsmIO {
     float* uzw;         // u(t + 1)
 };
 
-// ---- launchers (lbif_kernels.cu) -------------------------------------------
+// ---- launchers (lbif_kernels.cu, lbif_force.cu, lbif_pull.cu) ---------------
 cudaError_t launch_fill_outside(const Params& P, float* const* planes, const float* values,
                                 int nplanes, cudaStream_t s);
 // the initial states are equilibria: the caller zeroes the stored populations
