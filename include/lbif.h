@@ -262,7 +262,8 @@ int lbif_autotune(lbif_handle h, int32_t trials, int32_t* ball_want, int32_t* fo
                   int32_t* ball_staging);
 /* The launch shapes in use: shapes[0] ball CTA target (0 = default),
  * [1] force tile-group edge (0 = default), [2] ball staging (1 = tensor-
- * memory accelerator), [3] pull-pass z planes per segment (0 = default 16),
+ * memory accelerator), [3] pull-pass z planes per segment (0 = chosen from the
+ * grid's size),
  * [4] pull-pass gathers (0 plain, 1 prefetched, 2 tensor-memory accelerator). */
 int lbif_get_shapes(lbif_handle h, int32_t shapes[5]);
 /* Set the launch shapes (same order and meaning as lbif_get_shapes) instead of

@@ -32,6 +32,7 @@ namespace lbif {
 
 constexpr int Q = 19;
 constexpr int MAX_SIGMA = 24;
+constexpr int NUM_SMS = 152;  // GB300
 constexpr int PAD_SLACK = 64;  // floats before and after every padded array
 
 struct Geom {
@@ -166,9 +167,10 @@ cudaError_t tail_spectral_init(const Geom& g, int D, const int* pdx, const int* 
 cudaError_t launch_tail_spectral(const Params& P, const float* dn, int D, float2* work, float4* Ft,
                                  cudaStream_t s);
 // one step's collision, pull streaming and the moments of the new
-// populations (CsmIO); lz: z planes per CTA segment of the tiled kernel
-// (<= 0: default); prefetch: 0 plain, 1 the next plane's population gathers
-// issued before the current plane is collided, 2 the gathers brought in by
+// populations (CsmIO); lz: z planes per CTA segment of the tiled kernels
+// (<= 0: default); prefetch: 0 two planes per round with plain gathers, 1 one
+// plane per round, the next plane's population gathers issued before the
+// current plane is collided, 2 one plane per round, the gathers brought in by
 // the tensor-memory accelerator from pmap (a 4-D map of pin: x, y, z,
 // direction, box from pop_box; two-buffer layout only; bit 4 of status
 // records a bounded wait that ran out). Grids narrower than one tile run the

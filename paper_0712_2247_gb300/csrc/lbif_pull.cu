@@ -1,5 +1,7 @@
 // The pull pass: collision, streaming and the next step's moments in one pass
 // over the populations, with its launchers.
+#include <math.h>
+
 #include <atomic>
 #include <utility>
 
@@ -47,13 +49,40 @@ namespace lbif {
 template <typename T>
 __host__ __device__ constexpr float store_scale() { return sizeof(T) == 2 ? 256.f : 1.f; }
 
+// The pass's arithmetic, written once for one node (float) and for two nodes
+// at a time (float2: one fma / add / mul .f32x2 instruction does both, each
+// component rounding as the scalar operation). Every operation is explicit, so
+// all kernels of the pass give identical results. The compiler merges a paired
+// product into a paired addition that takes it (the scalar intrinsics it
+// leaves alone): a product that feeds an addition is therefore written as one
+// vfma, or rounded by itself as vfma(a, b, 0) (vprod).
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ float vrdiv(float a, float b) { return __fdiv_rn(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return add2(a, b); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return sub2(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return mul2(a, b); }
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 vrdiv(float a, float2 b) { return make_float2(__fdiv_rn(a, b.x), __fdiv_rn(a, b.y)); }
+template <class V>
+__device__ __forceinline__ V vset(float s);
+template <>
+__device__ __forceinline__ float vset<float>(float s) { return s; }
+template <>
+__device__ __forceinline__ float2 vset<float2>(float s) { return bc2(s); }
+
+template <class V>
+__device__ __forceinline__ V vprod(V a, V b) { return vfma(a, b, vset<V>(0.f)); }
+
 // staged quantities of a node: dn, P_x..z, C_x..z, C_xy C_xz C_yz, X_xy X_xz X_yz
 constexpr int SQ_DN = 0, SQ_P = 1, SQ_CA = 4, SQ_CP = 7, SQ_X = 10, CSM_NF = 13;
 
 // The staged quantities of a node from its moments and force; st(k, value)
-// receives quantity k. Each quantity ends in a rounding intrinsic (never
-// merged into a later multiply-add), so a kernel that uses them at once and
-// one that stores them first compute identical values.
+// receives quantity k; om = 1/tau is used by the shifted form only.
 //
 // shifted (velocity-shifted second-order forcing, the force F from the
 // unshifted moments): BGK towards f^eq(n, u') with u' = u + F/(2 q), and the
@@ -64,81 +93,111 @@ constexpr int SQ_DN = 0, SQ_P = 1, SQ_CA = 4, SQ_CP = 7, SQ_X = 10, CSM_NF = 13;
 //   alpha   = -(3/2) q ((1 - omega) u.u + omega u'.u') - 3 k u'.F
 //   beta_a  = 3 q ((1 - omega) u_a + omega u'_a) + 3 k F_a
 //   gamma_ab = (9/2) q ((1 - omega) u_a u_b + omega u'_a u'_b) + (9/2) k (u'_a F_b + u'_b F_a).
-template <class St>
-__device__ __forceinline__ void src_terms(float d, float ux, float uy, float uz, float4 f, float om, bool shifted,
-                                          St st)
+template <class V, class St>
+__device__ __forceinline__ void src_terms(V d, V ux, V uy, V uz, V fx, V fy, V fz, V fw, V om, bool shifted, St st)
 {
-    const float q1 = 1.f + d;
+    const V q1 = vadd(vset<V>(1.f), d);
     st(SQ_DN, d);
     if (shifted) {
-        const float hq = 0.5f / q1;
-        const float vx = fmaf(hq, f.x, ux), vy = fmaf(hq, f.y, uy), vz = fmaf(hq, f.z, uz);  // u'
-        const float k = fmaf(-0.5f, om, 1.f), a1 = 1.f - om;
-        const float uu = ux * ux + uy * uy + uz * uz, vv = vx * vx + vy * vy + vz * vz;
-        const float vF = vx * f.x + vy * f.y + vz * f.z;
-        const float alpha = fmaf(-1.5f * q1, fmaf(a1, uu, om * vv), -3.f * k * vF);
-        const float u[3] = {ux, uy, uz}, v[3] = {vx, vy, vz}, F[3] = {f.x, f.y, f.z};
+        const V hq = vrdiv(0.5f, q1);
+        const V u[3] = {ux, uy, uz}, F[3] = {fx, fy, fz};
+        const V v[3] = {vfma(hq, fx, ux), vfma(hq, fy, uy), vfma(hq, fz, uz)};  // u'
+        const V k = vfma(vset<V>(-0.5f), om, vset<V>(1.f)), a1 = vsub(vset<V>(1.f), om);
+        auto dot = [](const V* a, const V* b) { return vfma(a[2], b[2], vfma(a[1], b[1], vmul(a[0], b[0]))); };
+        const V k3 = vmul(vset<V>(3.f), k), k45 = vmul(vset<V>(4.5f), k), q45 = vmul(vset<V>(4.5f), q1);
+        const V alpha = vfma(vmul(vset<V>(-1.5f), q1), vfma(a1, dot(u, u), vmul(om, dot(v, v))),
+                             vmul(vset<V>(-1.f), vmul(k3, dot(v, F))));
         auto gam = [&](int a, int b) {
-            return fmaf(4.5f * q1, fmaf(a1, u[a] * u[b], om * (v[a] * v[b])), 4.5f * k * fmaf(v[a], F[b], v[b] * F[a]));
+            return vfma(q45, vfma(a1, vmul(u[a], u[b]), vmul(om, vmul(v[a], v[b]))),
+                        vmul(k45, vfma(v[a], F[b], vmul(v[b], F[a]))));
         };
-        const float gxx = gam(0, 0), gyy = gam(1, 1), gzz = gam(2, 2);
+        const V gxx = gam(0, 0), gyy = gam(1, 1), gzz = gam(2, 2);
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-            st(SQ_P + a, __fmul_rn(3.f, fmaf(q1, fmaf(a1, u[a], om * v[a]), k * F[a])));
-        st(SQ_CA + 0, __fadd_rn(alpha, gxx));
-        st(SQ_CA + 1, __fadd_rn(alpha, gyy));
-        st(SQ_CA + 2, __fadd_rn(alpha, gzz));
-        st(SQ_CP + 0, __fadd_rn(alpha, gxx + gyy));
-        st(SQ_CP + 1, __fadd_rn(alpha, gxx + gzz));
-        st(SQ_CP + 2, __fadd_rn(alpha, gyy + gzz));
-        st(SQ_X + 0, __fmul_rn(2.f, gam(0, 1)));
-        st(SQ_X + 1, __fmul_rn(2.f, gam(0, 2)));
-        st(SQ_X + 2, __fmul_rn(2.f, gam(1, 2)));
+            st(SQ_P + a, vmul(vset<V>(3.f), vfma(q1, vfma(a1, u[a], vmul(om, v[a])), vmul(k, F[a]))));
+        st(SQ_CA + 0, vadd(alpha, gxx));
+        st(SQ_CA + 1, vadd(alpha, gyy));
+        st(SQ_CA + 2, vadd(alpha, gzz));
+        st(SQ_CP + 0, vadd(alpha, vadd(gxx, gyy)));
+        st(SQ_CP + 1, vadd(alpha, vadd(gxx, gzz)));
+        st(SQ_CP + 2, vadd(alpha, vadd(gyy, gzz)));
+        st(SQ_X + 0, vmul(vset<V>(2.f), gam(0, 1)));
+        st(SQ_X + 1, vmul(vset<V>(2.f), gam(0, 2)));
+        st(SQ_X + 2, vmul(vset<V>(2.f), gam(1, 2)));
         return;
     }
-    const float B = __fmul_rn(-1.5f * q1, ux * ux + uy * uy + uz * uz);
-    const float a = 4.5f * q1, ax = a * ux * ux, ay = a * uy * uy, az = a * uz * uz;
-    const float fw = 1.5f * f.w, b = 9.f * q1;
-    st(SQ_P + 0, __fmul_rn(3.f, fmaf(q1, ux, f.x)));
-    st(SQ_P + 1, __fmul_rn(3.f, fmaf(q1, uy, f.y)));
-    st(SQ_P + 2, __fmul_rn(3.f, fmaf(q1, uz, f.z)));
-    st(SQ_CA + 0, __fadd_rn(B, ax));
-    st(SQ_CA + 1, __fadd_rn(B, ay));
-    st(SQ_CA + 2, __fadd_rn(B, az));
-    st(SQ_CP + 0, __fadd_rn(B + (ax + ay), fw));
-    st(SQ_CP + 1, __fadd_rn(B + (ax + az), fw));
-    st(SQ_CP + 2, __fadd_rn(B + (ay + az), fw));
-    st(SQ_X + 0, __fmul_rn(b * ux, uy));
-    st(SQ_X + 1, __fmul_rn(b * ux, uz));
-    st(SQ_X + 2, __fmul_rn(b * uy, uz));
+    const V uu = vfma(uz, uz, vfma(uy, uy, vmul(ux, ux)));
+    const V B = vmul(vmul(vset<V>(-1.5f), q1), uu);
+    const V a = vmul(vset<V>(4.5f), q1), aux = vmul(a, ux), auy = vmul(a, uy), auz = vmul(a, uz);
+    const V Cx = vfma(aux, ux, B), Cy = vfma(auy, uy, B), Cz = vfma(auz, uz, B), f15 = vset<V>(1.5f);
+    st(SQ_P + 0, vmul(vset<V>(3.f), vfma(q1, ux, fx)));
+    st(SQ_P + 1, vmul(vset<V>(3.f), vfma(q1, uy, fy)));
+    st(SQ_P + 2, vmul(vset<V>(3.f), vfma(q1, uz, fz)));
+    st(SQ_CA + 0, Cx);
+    st(SQ_CA + 1, Cy);
+    st(SQ_CA + 2, Cz);
+    st(SQ_CP + 0, vfma(f15, fw, vfma(auy, uy, Cx)));
+    st(SQ_CP + 1, vfma(f15, fw, vfma(auz, uz, Cx)));
+    st(SQ_CP + 2, vfma(f15, fw, vfma(auz, uz, Cy)));
+    const V bx = vmul(vset<V>(2.f), aux), by = vmul(vset<V>(2.f), auy);  // 9 q u_x, 9 q u_y
+    st(SQ_X + 0, vmul(bx, uy));
+    st(SQ_X + 1, vmul(bx, uz));
+    st(SQ_X + 2, vmul(by, uz));
 }
 
-// v_i (see above) from the source's staged quantities sl (quantity k at
-// sl[k * ST]) and its stored h; wall: sl is the node itself and the
-// direction arrives reversed
-template <int i, int ST>
-__device__ __forceinline__ float arrive(const float* sl, float h, float om1s, float dnr, bool wall)
+// C_0 of a node from its staged quantities (see above)
+template <class V>
+__device__ __forceinline__ V rest_term(V cx, V cy, V cz, V cxy, V cxz, V cyz)
+{
+    const V s = vadd(vadd(cx, cy), cz), d = vadd(vadd(cxy, cxz), cyz);
+    return vmul(vsub(vadd(s, s), d), vset<V>(1.f / 3.f));
+}
+
+// a node's staged quantities at p, quantity k at p[k ST]
+template <int ST>
+struct Strided {
+    const float* p;
+    template <int K>
+    __device__ __forceinline__ float get() const
+    {
+        return p[K * ST];
+    }
+    __device__ __forceinline__ float c0() const
+    {
+        return rest_term(get<SQ_CA>(), get<SQ_CA + 1>(), get<SQ_CA + 2>(), get<SQ_CP>(), get<SQ_CP + 1>(),
+                         get<SQ_CP + 2>());
+    }
+};
+
+// v_i (see above) from the source's staged quantities s and its stored h;
+// wall: s is the node itself and the direction arrives reversed
+template <int i, class V, class Src>
+__device__ __forceinline__ V arrive(const Src& s, V h, float om1s, V dnr, bool wall)
 {
     constexpr int cx = kCx(i), cy = kCy(i), cz = kCz(i);
-    const float sg = wall ? -1.f : 1.f;
-    float t;
+    const V o = vset<V>(om1s), ds = s.template get<SQ_DN>(), m = vfma(o, ds, o);
     if constexpr (i == 0) {
-        t = (2.f * (sl[(SQ_CA + 0) * ST] + sl[(SQ_CA + 1) * ST] + sl[(SQ_CA + 2) * ST]) -
-             (sl[(SQ_CP + 0) * ST] + sl[(SQ_CP + 1) * ST] + sl[(SQ_CP + 2) * ST])) *
-            (1.f / 3.f);
-    } else if constexpr (kC2(i) == 1) {
-        constexpr int a = cx ? 0 : (cy ? 1 : 2);
-        constexpr float ca = (float)(cx + cy + cz);
-        t = fmaf(sg * ca, sl[(SQ_P + a) * ST], sl[(SQ_CA + a) * ST]);
+        return vfma(m, h, s.c0());
     } else {
-        constexpr int pl = cz == 0 ? 0 : (cy == 0 ? 1 : 2);
-        constexpr int a = pl == 2 ? 1 : 0, b = pl == 0 ? 1 : 2;
-        constexpr float ca = (float)(a == 0 ? cx : cy), cb = (float)(b == 1 ? cy : cz);
-        t = sl[(SQ_CP + pl) * ST] + sg * (ca * sl[(SQ_P + a) * ST] + cb * sl[(SQ_P + b) * ST]) +
-            (ca * cb) * sl[(SQ_X + pl) * ST];
+        V p, t;
+        if constexpr (kC2(i) == 1) {
+            constexpr int a = cx ? 0 : (cy ? 1 : 2);
+            p = s.template get<SQ_P + a>();
+            t = s.template get<SQ_CA + a>();
+            t = (cx + cy + cz > 0) != wall ? vadd(t, p) : vsub(t, p);
+        } else {
+            constexpr int pl = cz == 0 ? 0 : (cy == 0 ? 1 : 2);
+            constexpr int a = pl == 2 ? 1 : 0, b = pl == 0 ? 1 : 2;
+            constexpr bool pa = (a == 0 ? cx : cy) > 0, same = pa == ((b == 1 ? cy : cz) > 0);
+            const V A = s.template get<SQ_P + a>(), B = s.template get<SQ_P + b>();
+            p = same ? vadd(A, B) : vsub(A, B);
+            t = s.template get<SQ_CP + pl>();
+            t = pa != wall ? vadd(t, p) : vsub(t, p);
+            const V X = s.template get<SQ_X + pl>();
+            t = same ? vadd(t, X) : vsub(t, X);
+        }
+        return vadd(vfma(m, h, t), vsub(ds, dnr));
     }
-    const float ds = sl[SQ_DN * ST];
-    return fmaf(fmaf(om1s, ds, om1s), h, t) + (ds - dnr);
 }
 
 // fn(std::integral_constant<int, i>) for i = 0 .. Q-1, unrolled at compile time
@@ -174,27 +233,30 @@ struct Mirror {
     static constexpr float CB = axis ? 0.f : (float)(B == 0 ? kCx(i) : (B == 1 ? kCy(i) : kCz(i)));
 };
 
-// v_i - v_ip of a mirror pair (staged quantities of the sources at s and sp,
-// stride ST; the stored values h, hp of the two directions; wall: both
-// arrive reversed from the node itself, s = sp)
-template <int i, int ip, int ST>
-__device__ __forceinline__ float mirror_diff(const float* s, const float* sp, float h, float hp, float om1s, bool wall)
+// v_i - v_ip of a mirror pair (staged quantities of the sources s and sp; the
+// stored values h, hp of the two directions; wall: both arrive reversed from
+// the node itself, s = sp)
+template <int i, int ip, class V, class Src>
+__device__ __forceinline__ V mirror_diff(const Src& s, const Src& sp, V h, V hp, float om1s, bool wall)
 {
     using M = Mirror<i, ip>;
-    const float sg = wall ? -1.f : 1.f;
-    float dt;
+    const V pa = vadd(s.template get<SQ_P + M::A>(), sp.template get<SQ_P + M::A>());
+    V dt;
     if constexpr (M::axis) {
-        dt = (s[(SQ_CA + M::A) * ST] - sp[(SQ_CA + M::A) * ST]) + sg * (s[(SQ_P + M::A) * ST] + sp[(SQ_P + M::A) * ST]);
+        dt = vsub(s.template get<SQ_CA + M::A>(), sp.template get<SQ_CA + M::A>());
+        dt = wall ? vsub(dt, pa) : vadd(dt, pa);
     } else {
-        dt = (s[(SQ_CP + M::PL) * ST] - sp[(SQ_CP + M::PL) * ST]) +
-             sg * (s[(SQ_P + M::A) * ST] + sp[(SQ_P + M::A) * ST]) +
-             (sg * M::CB) * (s[(SQ_P + M::B) * ST] - sp[(SQ_P + M::B) * ST]) +
-             M::CB * (s[(SQ_X + M::PL) * ST] + sp[(SQ_X + M::PL) * ST]);
+        dt = vsub(s.template get<SQ_CP + M::PL>(), sp.template get<SQ_CP + M::PL>());
+        dt = wall ? vsub(dt, pa) : vadd(dt, pa);
+        const V pb = vsub(s.template get<SQ_P + M::B>(), sp.template get<SQ_P + M::B>());
+        dt = (M::CB > 0.f) != wall ? vadd(dt, pb) : vsub(dt, pb);
+        const V X = vadd(s.template get<SQ_X + M::PL>(), sp.template get<SQ_X + M::PL>());
+        dt = M::CB > 0.f ? vadd(dt, X) : vsub(dt, X);
     }
-    const float ds = s[SQ_DN * ST], dsp = sp[SQ_DN * ST];
+    const V ds = s.template get<SQ_DN>(), dd = vsub(ds, sp.template get<SQ_DN>());
     // m(s) h - m(sp) hp with m = om1s (1 + d)
-    const float dm = om1s * fmaf(1.f + ds, h - hp, (ds - dsp) * hp);
-    return (dt + dm) + (ds - dsp);
+    const V dm = vfma(vadd(vset<V>(1.f), ds), vsub(h, hp), vmul(dd, hp));
+    return vadd(vfma(vset<V>(om1s), dm, dt), dd);
 }
 
 // element off of direction i's part of a population buffer
@@ -213,66 +275,65 @@ __device__ __forceinline__ T* pop_at_ip(T* p, const Params& P, int i, int slot)
 
 // the new moments of a node from its arriving values (slots as above, d79 =
 // v_7 - v_9), then its populations stored as non-equilibrium parts at those
-// moments (at(i): where direction i goes): base directions directly, derived
-// ones as their partner's stored value plus the difference (so the pairs'
-// differences survive the rounding of the large common parts); returns dn
-// and writes u
-template <typename T, class Addr>
-__device__ __forceinline__ float pull_finish(Addr at, const float* v, float d79, float dnr, float& ux, float& uy,
-                                             float& uz)
+// moments (put(i, h)): base directions directly, derived ones as their
+// partner's stored value plus the difference (so the pairs' differences
+// survive the rounding of the large common parts); returns dn and writes u
+template <typename T, class V, class Put>
+__device__ __forceinline__ V pull_finish(Put put, const V* v, V d79, V dnr, V& ux, V& uy, V& uz)
 {
-    constexpr float w1 = 1.f / 18.f, w2 = 1.f / 36.f;
+    const V w1 = vset<V>(1.f / 18.f), w2 = vset<V>(1.f / 36.f);
     // arriving values of the derived directions
-    const float v1 = v[2] + v[1], v3 = v[4] + v[3], v9 = v[8] + v[9], v10 = v[8] + v[10];
-    const float v7 = v10 + v[7], v11 = v[14] + v[11], v13 = v[12] + v[13], v15 = v[18] + v[15];
-    const float v17 = v[16] + v[17];
-    const float S = (1.f / 3.f) * v[0] +
-                    w1 * (((v1 + v[2]) + (v3 + v[4])) + (v[5] + v[6])) +
-                    w2 * ((((v7 + v[8]) + (v9 + v10)) + ((v11 + v[12]) + (v13 + v[14]))) +
-                          ((v15 + v[16]) + (v17 + v[18])));
-    const float Jz = w1 * (v[5] - v[6]) +
-                     w2 * (((v11 - v[12]) - (v13 - v[14])) + ((v15 - v[16]) - (v17 - v[18])));
-    const float Jx = w1 * v[1] + w2 * (((v[7] + v[9]) + (v[11] + v[13])));
-    const float Jy = w1 * v[3] + w2 * ((d79 + v[10]) + (v[15] + v[17]));
-    const float dn = dnr + S;
-    const float inv = 1.f / (1.f + dn);
-    ux = Jx * inv;
-    uy = Jy * inv;
-    uz = Jz * inv;
-    const float uu = ux * ux + uy * uy + uz * uz;
-    constexpr float sT = store_scale<T>();
-    auto p_of = [&](int i) {  // f_i^eq / (w_i n) - 1
-        const float cu = dot_c(i, ux, uy, uz);
-        return fmaf(cu, fmaf(4.5f, cu, 3.f), -1.5f * uu);
+    const V v1 = vadd(v[2], v[1]), v3 = vadd(v[4], v[3]), v9 = vadd(v[8], v[9]), v10 = vadd(v[8], v[10]);
+    const V v7 = vadd(v10, v[7]), v11 = vadd(v[14], v[11]), v13 = vadd(v[12], v[13]), v15 = vadd(v[18], v[15]);
+    const V v17 = vadd(v[16], v[17]);
+    const V sa = vadd(vadd(vadd(v1, v[2]), vadd(v3, v[4])), vadd(v[5], v[6]));
+    const V sd = vadd(vadd(vadd(vadd(v7, v[8]), vadd(v9, v10)), vadd(vadd(v11, v[12]), vadd(v13, v[14]))),
+                      vadd(vadd(v15, v[16]), vadd(v17, v[18])));
+    const V S = vfma(w2, sd, vfma(w1, sa, vmul(vset<V>(1.f / 3.f), v[0])));
+    const V jz = vadd(vsub(vsub(v11, v[12]), vsub(v13, v[14])), vsub(vsub(v15, v[16]), vsub(v17, v[18])));
+    const V Jz = vfma(w2, jz, vmul(w1, vsub(v[5], v[6])));
+    const V Jx = vfma(w2, vadd(vadd(v[7], v[9]), vadd(v[11], v[13])), vmul(w1, v[1]));
+    const V Jy = vfma(w2, vadd(vadd(d79, v[10]), vadd(v[15], v[17])), vmul(w1, v[3]));
+    const V dn = vadd(dnr, S);
+    const V inv = vrdiv(1.f, vadd(vset<V>(1.f), dn));
+    ux = vprod(Jx, inv);
+    uy = vprod(Jy, inv);
+    uz = vprod(Jz, inv);
+    const V u15 = vmul(vset<V>(1.5f), vfma(uz, uz, vfma(uy, uy, vmul(ux, ux))));
+    const V sT = vset<V>(store_scale<T>());
+    auto store = [&](int i, V h) { put(i, sizeof(T) == 2 ? vmul(sT, h) : h); };
+    // (v_i - S) / (1 + dn) - p_i with p_i = f_i^eq / (w_i n) - 1 =
+    // c.u (3 + 9/2 c.u) - 3/2 u.u, of a base direction with cm = -c.u
+    auto base = [&](V vi, V cm) {
+        return vfma(vsub(vi, S), inv, vfma(cm, vfma(vset<V>(-4.5f), cm, vset<V>(3.f)), u15));
     };
-    auto base = [&](int i, float vi) { return (vi - S) * inv - p_of(i); };
-    // p_i - p_ip of a pair that differs in component a: u_a (6 + 18 R),
-    // R = the shared part of c.u
-    auto dp = [&](float ua, float R) { return ua * fmaf(18.f, R, 6.f); };
-    auto put = [&](int i, float h) { stp(at(i), sT * h); };
-    put(0, base(0, v[0]));
-    put(5, base(5, v[5]));
-    put(6, base(6, v[6]));
-    const float h2 = base(2, v[2]), h4 = base(4, v[4]), h8 = base(8, v[8]);
-    put(2, h2);
-    put(1, h2 + (v[1] * inv - dp(ux, 0.f)));
-    put(4, h4);
-    put(3, h4 + (v[3] * inv - dp(uy, 0.f)));
-    put(8, h8);
-    put(9, h8 + (v[9] * inv - dp(ux, -uy)));
-    const float h10 = h8 + (v[10] * inv - dp(uy, -ux));
-    put(10, h10);
-    put(7, h10 + (v[7] * inv - dp(ux, uy)));
-    const float h12 = base(12, v[12]), h14 = base(14, v[14]);
-    put(12, h12);
-    put(13, h12 + (v[13] * inv - dp(ux, -uz)));
-    put(14, h14);
-    put(11, h14 + (v[11] * inv - dp(ux, uz)));
-    const float h16 = base(16, v[16]), h18 = base(18, v[18]);
-    put(16, h16);
-    put(17, h16 + (v[17] * inv - dp(uy, -uz)));
-    put(18, h18);
-    put(15, h18 + (v[15] * inv - dp(uy, uz)));
+    // v inv - (p_i - p_ip) of a pair that differs in component a:
+    // p_i - p_ip = u_a (6 + 18 R), R = the shared part of c.u (Rm = -R)
+    auto diff = [&](V vi, V ua, V Rm) { return vfma(vi, inv, vmul(ua, vfma(vset<V>(18.f), Rm, vset<V>(-6.f)))); };
+    const V six = vset<V>(-6.f);
+    store(0, vfma(vsub(v[0], S), inv, u15));
+    store(5, base(v[5], vneg(uz)));
+    store(6, base(v[6], uz));
+    const V h2 = base(v[2], ux), h4 = base(v[4], uy), h8 = base(v[8], vadd(ux, uy));
+    store(2, h2);
+    store(1, vadd(h2, vfma(v[1], inv, vmul(ux, six))));
+    store(4, h4);
+    store(3, vadd(h4, vfma(v[3], inv, vmul(uy, six))));
+    store(8, h8);
+    store(9, vadd(h8, diff(v[9], ux, uy)));
+    const V h10 = vadd(h8, diff(v[10], uy, ux));
+    store(10, h10);
+    store(7, vadd(h10, diff(v[7], ux, vneg(uy))));
+    const V h12 = base(v[12], vadd(ux, uz)), h14 = base(v[14], vsub(ux, uz));
+    store(12, h12);
+    store(13, vadd(h12, diff(v[13], ux, uz)));
+    store(14, h14);
+    store(11, vadd(h14, diff(v[11], ux, vneg(uz))));
+    const V h16 = base(v[16], vadd(uy, uz)), h18 = base(v[18], vsub(uy, uz));
+    store(16, h16);
+    store(17, vadd(h16, diff(v[17], uy, uz)));
+    store(18, h18);
+    store(15, vadd(h18, diff(v[15], uy, vneg(uz))));
     return dn;
 }
 
@@ -294,12 +355,12 @@ __device__ __forceinline__ void put_fields(const Params& P, const CsmIO& io, int
 }
 
 // What a source node contributes is staged per node in shared memory: a CTA
-// owns a 32 x 4 tile of x-y nodes, keeps three planes of it (plus a one-node
-// halo) in a ring, and marches up a segment of z planes.
-// 32 x 4 tiles of 128 threads, six CTAs per SM (measured at 512 x 512 x 192, sigma 12, same
-// state: 32 x 4 / 128 threads / 6 CTAs 2.186 ms, 32 x 8 / 256 / 3 2.334 ms, 32 x 12 / 384 / 2
-// 2.508 ms): more, smaller CTAs keep more population loads in flight across the two barriers
-// of each plane
+// owns a 32 x 4 tile of x-y nodes (more, smaller CTAs keep more population
+// loads in flight across the two barriers of a round: 32 x 8 and 32 x 12 tiles
+// ran 7 % and 15 % slower) and marches it up a segment of z planes. Three
+// forms: two planes per round (the default, k_pull_pair below), and one plane
+// per round with the next plane's gathers issued early (k_csm) or copied by
+// the tensor-memory accelerator (k_csm_tma), whose ring holds three planes.
 constexpr int CSM_TX = 32, CSM_TY = 4, CSM_THREADS = CSM_TX * CSM_TY;
 constexpr int CSM_HX = CSM_TX + 2, CSM_HN = CSM_HX * (CSM_TY + 2);  // staged nodes per plane
 constexpr int CSM_SLOT = CSM_NF * CSM_HN;  // floats per staged plane
@@ -358,20 +419,16 @@ __device__ __forceinline__ void csm_stage(const Params& P, const CsmIO& io, cons
         if (k * NT >= CSM_HN || st.p[k] < 0) continue;
         const int h = threadIdx.x + k * NT;
         const int p = pq + st.p[k];
-        src_terms(__ldg(io.dn + p), __ldg(io.ux + p), __ldg(io.uy + p), __ldg(io.uz + p), __ldg(Fq + st.n[k]), om,
+        const float4 f = __ldg(Fq + st.n[k]);
+        src_terms(__ldg(io.dn + p), __ldg(io.ux + p), __ldg(io.uy + p), __ldg(io.uz + p), f.x, f.y, f.z, f.w, om,
                   shifted, [&](int j, float val) { slot[j * CSM_HN + h] = val; });
     }
 }
 
-// CTAs per SM the register budget is sized for (5 / 6 / 7 at 96 / 80 / 72
-// registers: 2.57 / 2.39 / 2.55 ms at 512 x 512 x 192, sigma 12, FP32), and
-// z planes per CTA segment
-#ifndef CSM_MINB
-#define CSM_MINB 6
-#endif
-#ifndef CSM_LZ
-#define CSM_LZ 16
-#endif
+// CTAs per SM the register budget of the one-plane forms is sized for, and
+// their z planes per CTA segment
+constexpr int CSM_MINB = 5;
+constexpr int CSM_LZ = 16;
 
 // the stored populations of directions [I0, I1) that stream into node
 // (x, y, z): v[i - I0]; bit i of bb marks a direction that arrives from a
@@ -416,24 +473,27 @@ __device__ __forceinline__ void csm_pull(const Params& P, const T* __restrict__ 
     }
 }
 
-// The arriving values of a node in the slots described at Mirror: the ten
-// mirror differences first (from the stored values as loaded), then the ten
-// base directions. src(i) is the source quantities of direction i (stride
-// ST); wall directions arrive reversed from the node itself (own).
-template <int ST, bool WALLS, class Src>
-__device__ __forceinline__ void pull_gather_impl(Src src, const float* own, float om1s, float dnr, unsigned bb,
-                                                 float* v, float& d79)
+// The arriving values of a node (or a pair of nodes) in the slots described
+// at Mirror: the ten mirror differences first (from the stored values as
+// loaded), then the ten base directions. src(i) is the source quantities of
+// direction i; wall directions (bit i of bb) arrive reversed from the node
+// itself (own).
+template <bool WALLS, class V, class SrcOf, class Own>
+__device__ __forceinline__ void pull_gather_impl(SrcOf src, const Own& own, float om1s, V dnr, unsigned bb, V* v,
+                                                 V& d79)
 {
     auto wall = [&](int i) { return WALLS && ((bb >> i) & 1u) != 0u; };
-    auto diff = [&](auto ic, auto ipc) {
+    auto diff = [&](auto ic, auto ipc) -> V {
         constexpr int i = decltype(ic)::value, ip = decltype(ipc)::value;
-        const bool w = wall(i);
-        return mirror_diff<i, ip, ST>(w ? own : src(ic), w ? own : src(ipc), v[i], v[ip], om1s, w);
+        if constexpr (WALLS && kCz(i) != 0) {
+            if (wall(i)) return mirror_diff<i, ip, V>(own, own, v[i], v[ip], om1s, true);
+        }
+        return mirror_diff<i, ip, V>(src(ic), src(ipc), v[i], v[ip], om1s, false);
     };
     using std::integral_constant;
-    const float d7_10 = diff(integral_constant<int, 7>{}, integral_constant<int, 10>{});
-    const float d9_8 = diff(integral_constant<int, 9>{}, integral_constant<int, 8>{});
-    const float d10_8 = diff(integral_constant<int, 10>{}, integral_constant<int, 8>{});
+    const V d7_10 = diff(integral_constant<int, 7>{}, integral_constant<int, 10>{});
+    const V d9_8 = diff(integral_constant<int, 9>{}, integral_constant<int, 8>{});
+    const V d10_8 = diff(integral_constant<int, 10>{}, integral_constant<int, 8>{});
     d79 = diff(integral_constant<int, 7>{}, integral_constant<int, 9>{});
     v[7] = d7_10;
     v[9] = d9_8;
@@ -446,57 +506,54 @@ __device__ __forceinline__ void pull_gather_impl(Src src, const float* own, floa
     v[17] = diff(integral_constant<int, 17>{}, integral_constant<int, 16>{});
     auto one = [&](auto ic) {
         constexpr int i = decltype(ic)::value;
-        if constexpr (i == 0 || i == 2 || i == 4 || i == 5 || i == 6 || i == 8 || i == 12 || i == 14 || i == 16 ||
-                      i == 18) {
-            const bool w = i != 0 && wall(i);
-            v[i] = arrive<i, ST>((i == 0 || w) ? own : src(ic), v[i], om1s, dnr, w);
+        if constexpr (i == 0) {
+            v[i] = arrive<i, V>(own, v[i], om1s, dnr, false);
+        } else if constexpr (i == 2 || i == 4 || i == 5 || i == 6 || i == 8 || i == 12 || i == 14 || i == 16 ||
+                             i == 18) {
+            if constexpr (WALLS && kCz(i) != 0) {
+                if (wall(i)) {
+                    v[i] = arrive<i, V>(own, v[i], om1s, dnr, true);
+                    return;
+                }
+            }
+            v[i] = arrive<i, V>(src(ic), v[i], om1s, dnr, false);
         }
     };
     for_dirs(one);
 }
 
-// The arriving values of a node in the slots described at Mirror: the ten
-// mirror differences first (from the stored values as loaded), then the ten
-// base directions. src(i) is the source quantities of direction i (stride
-// ST); wall directions arrive reversed from the node itself (own). Nodes
-// with no wall direction (bb = 0, almost all) take a path without the wall
-// selections.
-template <int ST, class Src>
-__device__ __forceinline__ void pull_gather(Src src, const float* own, float om1s, float dnr, unsigned bb, float* v,
-                                            float& d79)
+// the same; nodes with no wall direction (bb = 0, almost all) take a path
+// without the wall selections
+template <class V, class SrcOf, class Own>
+__device__ __forceinline__ void pull_gather(SrcOf src, const Own& own, float om1s, V dnr, unsigned bb, V* v, V& d79)
 {
     if (bb == 0u)
-        pull_gather_impl<ST, false>(src, own, om1s, dnr, bb, v, d79);
+        pull_gather_impl<false, V>(src, own, om1s, dnr, bb, v, d79);
     else
-        pull_gather_impl<ST, true>(src, own, om1s, dnr, bb, v, d79);
+        pull_gather_impl<true, V>(src, own, om1s, dnr, bb, v, d79);
 }
 
 // the gather of a node staged at hc in the ring (planes below, own, above)
 __device__ __forceinline__ void csm_collide(const float* own, const float* below, const float* above, int hc,
                                             float om1s, float dnr, unsigned bb, float* v, float& d79)
 {
-    auto src = [&](auto ic) -> const float* {
+    using Src = Strided<CSM_HN>;
+    auto src = [&](auto ic) {
         constexpr int i = decltype(ic)::value;
         constexpr int cx = kCx(i), cy = kCy(i), cz = kCz(i);
-        return (cz > 0 ? below : (cz < 0 ? above : own)) + hc - cx - cy * CSM_HX;
+        return Src{(cz > 0 ? below : (cz < 0 ? above : own)) + hc - cx - cy * CSM_HX};
     };
-    pull_gather<CSM_HN>(src, own + hc, om1s, dnr, bb, v, d79);
+    pull_gather(src, Src{own + hc}, om1s, dnr, bb, v, d79);
 }
 
-// one node per thread, a CTA per 32 x 4 tile and z segment (measured with the
-// earlier storage: two threads per node, each gathering half of the
-// directions and adding the partial moments through shared memory, ran
-// slower at twice the warps). PF: the population gathers of the next plane
-// are issued before the current plane is staged and collided, so they are in
-// flight across both barriers (19 more live registers: five CTAs per SM).
-// FP16 gathers stay raw until the collision (measured at 512 x 512 x 192,
-// sigma 12: 2.71 -> 2.54 ms; on a 256-slit ensemble 0.388 -> 0.335 ms): the
-// staging between the gathers and their use then hides their latency, as it
-// does for FP32 values, which nothing touches before the collision
+// The prefetched form: one node per thread, the population gathers of the next
+// plane issued before the current plane is staged and collided, so they are in
+// flight across both barriers (96 registers, five CTAs per SM). FP16 gathers
+// stay raw until the collision, so that the staging hides their latency.
 template <typename T>
 constexpr bool F16_RAW = sizeof(T) == 2;
-template <typename T, bool PF, bool IP>
-__global__ void __launch_bounds__(CSM_THREADS, PF ? CSM_MINB - 1 : CSM_MINB)
+template <typename T, bool IP>
+__global__ void __launch_bounds__(CSM_THREADS, CSM_MINB)
     k_csm(Params P, const T* pin, T* pout, CsmIO io, const float4* __restrict__ F, int lz, int tiles_x, int tiles_y,
           int* status)
 {
@@ -513,43 +570,34 @@ __global__ void __launch_bounds__(CSM_THREADS, PF ? CSM_MINB - 1 : CSM_MINB)
     const int zb = seg * lz, ze = min(zb + lz, g.nz);
     const CsmStaged st = csm_staged<NT>(g, x0, y0);
     // the population gathers of plane z (act: the node steps; om its 1/tau)
-    // (in place, q returns the node's slots, which its stores reuse)
-    auto gather = [&](int z, float* v, unsigned& bb, bool& act, float& om, IpSlots& q) {
+    auto gather = [&](int z, float* v, unsigned& bb, bool& act, float& om) {
         const int s = slit_of(P, z);
         act = in_xy && s >= 0 && !frozen(P, s);
         bb = 0;
         om = 0.f;
         if (act) {
             om = P.sl[s].inv_tau;
+            IpSlots q;
             if constexpr (IP) q = ip_slots(P, P.sl[s], s, x, y, z);
             csm_pull<0, Q, IP, T, F16_RAW<T>>(P, pin, ((long long)z * g.ny + y) * g.nx + x, x, y, z, P.sl[s].zlo,
                                               P.sl[s].zhi, v, bb, q);
         }
     };
-    IpSlots qn, qz;
     float vn[Q];
-    unsigned bbn = 0;
-    bool actn = false;
-    float omn = 0.f;
-    if constexpr (PF) gather(zb, vn, bbn, actn, omn, qn);
+    unsigned bbn;
+    bool actn;
+    float omn;
+    gather(zb, vn, bbn, actn, omn);
     csm_stage<NT>(P, io, F, sm + csm_slot(zb - 1) * CSM_SLOT, st, zb - 1);
     csm_stage<NT>(P, io, F, sm + csm_slot(zb) * CSM_SLOT, st, zb);
     for (int z = zb; z < ze; ++z) {
-        // issue the population loads first: they do not depend on the ring
         float v[Q];
-        unsigned bb;
-        bool act;
-        float om;
-        if constexpr (PF) {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) v[i] = vn[i];
-            bb = bbn;
-            act = actn;
-            om = omn;
-            if (z + 1 < ze) gather(z + 1, vn, bbn, actn, omn, qn);
-        } else {
-            gather(z, v, bb, act, om, qz);
-        }
+        for (int i = 0; i < Q; ++i) v[i] = vn[i];
+        const unsigned bb = bbn;
+        const bool act = actn;
+        const float om = omn;
+        if (z + 1 < ze) gather(z + 1, vn, bbn, actn, omn);
         __syncthreads();  // the slot of plane z - 2 is free
         csm_stage<NT>(P, io, F, sm + csm_slot(z + 1) * CSM_SLOT, st, z + 1);
         __syncthreads();
@@ -567,21 +615,346 @@ __global__ void __launch_bounds__(CSM_THREADS, PF ? CSM_MINB - 1 : CSM_MINB)
         float ux, uy, uz;
         float dn;
         if constexpr (IP) {
-            // FP16: the stores reuse the gather's slots (2.64 -> 2.47 ms at
-            // 512 x 512 x 192, sigma 12); FP32 recomputes them (holding them
-            // across the collision spills there: 2.50 -> 2.57 ms)
-            IpSlots q;
-            if constexpr (PF || sizeof(T) == 4) {
-                const int s = slit_of(P, z);
-                q = ip_slots(P, P.sl[s], s, x, y, z);
-            } else {
-                q = qz;
-            }
-            dn = pull_finish<T>([&](int i) { return pop_at_ip(pout, P, i, q.slot(i)); }, v, d79, dnr, ux, uy, uz);
+            const int s = slit_of(P, z);
+            const IpSlots q = ip_slots(P, P.sl[s], s, x, y, z);
+            dn = pull_finish<T>([&](int i, float h) { stp(pop_at_ip(pout, P, i, q.slot(i)), h); }, v, d79, dnr, ux, uy,
+                                uz);
         } else {
-            dn = pull_finish<T>([&](int i) { return pop_at(pout, P, i, idx); }, v, d79, dnr, ux, uy, uz);
+            dn = pull_finish<T>([&](int i, float h) { stp(pop_at(pout, P, i, idx), h); }, v, d79, dnr, ux, uy, uz);
         }
         put_fields(P, io, x, y, z, dn, ux, uy, uz, status);
+    }
+}
+
+// ---- two planes at a time ------------------------------------------------
+// The default form: a thread owns the nodes (x, y, z) and (x, y, z + 1) and a
+// CTA marches its 32 x 4 tile up two planes per round. The pair's arithmetic
+// is paired FP32 (one instruction for both nodes), one shared-memory load
+// brings a staged quantity of both nodes, their wrapped x-y offsets are
+// computed once, and a round of two planes costs two barriers. Populations
+// stay scalar loads (one per node and direction), so the form has no
+// alignment condition and serves both storage layouts. Against one plane per
+// round and thread (the former default): 690 instructions per node for 1261,
+// and at 512 x 512 x 192, sigma 12, 2.39 -> 2.19 ms FP32 (0.66 of the copy
+// bandwidth at 196 B/node), 2.54 -> 1.90 ms FP16, 2.50 -> 2.34 ms FP32 in
+// place; 256 stacked slits FP16 in place 0.68 -> 0.59 ms. It waits on load
+// latency (14 warps per SM, 37 % issue): four CTAs per SM by registers (128)
+// and shared memory. Tried and slower: three CTAs with the next round's
+// gathers held in registers (2.32 ms), five CTAs at 96 registers (3.0 ms),
+// prefetching the next round's rows to L2 (2.11-2.27 ms FP32 by what it
+// spills, 1.93-2.13 ms FP16).
+//
+// Staged pairs (float2 per node of the halo tile). Of a round's planes
+// z - 1 .. z + 2 the populations with c_z = +1 come from (z - 1, z), those
+// with c_z = -1 from (z + 1, z + 2) and the others from (z, z + 1):
+//   AB[2]  nine quantities of the pairs (z - 1, z) and (z + 1, z + 2), the
+//          latter being the next round's former
+//   OW[2]  five quantities of the pair (z, z + 1) that only c_z = 0 asks for
+//          (C_x, C_y, C_xy, X_xy, C_0); its dn, P_x, P_y are read from AB
+// A round stages planes z + 1 and z + 2: the pair into AB, plane z + 1 as the
+// second half of this round's OW and plane z + 2 as the first half of the
+// next round's.
+constexpr int AB_DN = 0, AB_P = 1, AB_CZ = 4, AB_CP = 5, AB_X = 7, AB_NF = 9;  // P x y z; CP, X of xz, yz
+constexpr int OW_C = 0, OW_CP = 2, OW_X = 3, OW_C0 = 4, OW_NF = 5;
+constexpr int PAIR_FLOATS = 2 * CSM_HN * 2 * (AB_NF + OW_NF);
+constexpr int PAIR_MINB = 4;  // CTAs per SM
+
+__host__ __device__ constexpr int ab_of(int k)
+{
+    return k == SQ_DN ? AB_DN : (k < SQ_CA ? AB_P + (k - SQ_P) : (k == SQ_CA + 2 ? AB_CZ : (k < SQ_X ? AB_CP + (k - SQ_CP - 1) : AB_X + (k - SQ_X - 1))));
+}
+__host__ __device__ constexpr bool in_ow(int k) { return k == SQ_CA || k == SQ_CA + 1 || k == SQ_CP || k == SQ_X; }
+__host__ __device__ constexpr int ow_of(int k) { return k == SQ_CP ? OW_CP : (k == SQ_X ? OW_X : OW_C + (k - SQ_CA)); }
+
+// the staged pair of a round at one halo node, for the directions with c_z != 0
+struct SideSrc {
+    const float2* ab;
+    template <int K>
+    __device__ __forceinline__ float2 get() const
+    {
+        return ab[ab_of(K) * CSM_HN];
+    }
+};
+// and for those with c_z = 0: lo, hi = AB of (z - 1, z) and (z + 1, z + 2)
+struct LevelSrc {
+    const float2* ow;
+    const float2* lo;
+    const float2* hi;
+    template <int K>
+    __device__ __forceinline__ float2 get() const
+    {
+        if constexpr (in_ow(K))
+            return ow[ow_of(K) * CSM_HN];
+        else
+            return make_float2(lo[ab_of(K) * CSM_HN].y, hi[ab_of(K) * CSM_HN].x);
+    }
+    __device__ __forceinline__ float2 c0() const { return ow[OW_C0 * CSM_HN]; }
+};
+// one node j of the round's pair (the rounds that touch a wall, or where only
+// one of the two planes steps): sources beside it, below or above it, and itself
+struct LoneSrc {
+    const float* ow;   // component j of OW
+    const float* own;  // its plane in AB (z: second half of lo; z + 1: first half of hi)
+    const float* side; // the plane asked for (own, or the one below / above)
+    template <int K>
+    __device__ __forceinline__ float get() const
+    {
+        return in_ow(K) ? ow[2 * ow_of(K) * CSM_HN] : side[2 * ab_of(K) * CSM_HN];
+    }
+    __device__ __forceinline__ float c0() const { return ow[2 * OW_C0 * CSM_HN]; }
+};
+
+// the staging loads of planes q and q + 1 for one halo node, and what they become
+struct PairStage {
+    float2 d, ux, uy, uz;
+    float4 f0, f1;
+};
+
+// where direction i's populations are read from and written to, as pointers a
+// 32-bit node offset is added to (two buffers: src folds in -c_z planes)
+struct PullPtrs {
+    const void* src[Q];
+    void* dst[Q];
+};
+
+template <typename T, bool IP>
+__global__ void __launch_bounds__(CSM_THREADS, PAIR_MINB)
+    k_pull_pair(Params P, PullPtrs pp, CsmIO io, const float4* __restrict__ F, int lz, int tiles_x, int tiles_y,
+                int* status)
+{
+    constexpr int NT = CSM_THREADS;
+    constexpr bool RAW = F16_RAW<T>;
+    extern __shared__ __align__(16) float2 psm[];
+    float2* const AB = psm;
+    float2* const OW = psm + 2 * AB_NF * CSM_HN;
+    const Geom& g = P.g;
+    const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
+    const int tiles = tiles_x * tiles_y;
+    const int tile = blockIdx.x % tiles, seg = blockIdx.x / tiles;
+    const int x0 = (tile % tiles_x) * CSM_TX, y0 = (tile / tiles_x) * CSM_TY;
+    const int t = threadIdx.x;
+    const int x = x0 + t % CSM_TX, y = y0 + t / CSM_TX;
+    const int hc = (t / CSM_TX + 1) * CSM_HX + t % CSM_TX + 1;
+    const bool in_xy = x < nx && y < ny;
+    const int zb = seg * lz, ze = min(zb + lz, nz);
+    const CsmStaged st = csm_staged<NT>(g, x0, y0);
+    const int pplane = g.py * g.px;
+    const bool shifted = P.shifted != 0;
+
+    // plane q as stored (periodic image), -1 where nothing is staged
+    auto plane_of = [&](int q) -> int {
+        if (g.zper) q = q < 0 ? q + nz : (q >= nz ? q - nz : q);
+        if (q < 0 || q >= nz) return -1;
+        const int s = slit_of(P, q);
+        return s < 0 || frozen(P, s) ? -1 : q;
+    };
+    auto stage_load = [&](int q, int k, PairStage& a) {
+        a.d = a.ux = a.uy = a.uz = make_float2(0.f, 0.f);
+        a.f0 = a.f1 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k * NT >= CSM_HN || st.p[k] < 0) return;
+        const int p = (q + g.hw) * pplane + st.p[k];
+        const int q0 = plane_of(q), q1 = plane_of(q + 1);
+        if (q0 >= 0) {
+            a.d.x = __ldg(io.dn + p);
+            a.ux.x = __ldg(io.ux + p);
+            a.uy.x = __ldg(io.uy + p);
+            a.uz.x = __ldg(io.uz + p);
+            a.f0 = __ldg(F + (unsigned)(q0 * nxy + st.n[k]));
+        }
+        if (q1 >= 0) {
+            a.d.y = __ldg(io.dn + p + pplane);
+            a.ux.y = __ldg(io.ux + p + pplane);
+            a.uy.y = __ldg(io.uy + p + pplane);
+            a.uz.y = __ldg(io.uz + p + pplane);
+            a.f1 = __ldg(F + (unsigned)(q1 * nxy + st.n[k]));
+        }
+    };
+    // planes (q, q + 1) into pair slot ab; plane q completes own slot ow, plane
+    // q + 1 begins the other
+    auto stage_store = [&](int q, int k, const PairStage& a, int ab, int ow) {
+        if (k * NT >= CSM_HN || st.p[k] < 0) return;
+        const int h = t + k * NT;
+        float2 om = make_float2(0.f, 0.f);
+        if (shifted) {
+            const int q0 = plane_of(q), q1 = plane_of(q + 1);
+            if (q0 >= 0) om.x = P.sl[slit_of(P, q0)].inv_tau;
+            if (q1 >= 0) om.y = P.sl[slit_of(P, q1)].inv_tau;
+        }
+        float2* A = AB + ab * AB_NF * CSM_HN + h;
+        float2* O0 = OW + ow * OW_NF * CSM_HN + h;
+        float2* O1 = OW + (ow ^ 1) * OW_NF * CSM_HN + h;
+        float2 C[6];
+        src_terms(a.d, a.ux, a.uy, a.uz, make_float2(a.f0.x, a.f1.x), make_float2(a.f0.y, a.f1.y),
+                  make_float2(a.f0.z, a.f1.z), make_float2(a.f0.w, a.f1.w), om, shifted, [&](int j, float2 v) {
+                      if (j >= SQ_CA && j < SQ_X) C[j - SQ_CA] = v;
+                      if (in_ow(j)) {
+                          O0[ow_of(j) * CSM_HN].y = v.x;
+                          O1[ow_of(j) * CSM_HN].x = v.y;
+                      } else {
+                          A[ab_of(j) * CSM_HN] = v;
+                      }
+                  });
+        const float2 c0 = rest_term(C[0], C[1], C[2], C[3], C[4], C[5]);
+        O0[OW_C0 * CSM_HN].y = c0.x;
+        O1[OW_C0 * CSM_HN].x = c0.y;
+    };
+    {
+        PairStage a;
+        stage_load(zb - 1, 0, a);
+        stage_store(zb - 1, 0, a, 0, 1);
+        stage_load(zb - 1, 1, a);
+        stage_store(zb - 1, 1, a, 0, 1);
+    }
+    int xo[3], yo[3];  // x and y nx of the nodes' sources with c = 0, +1, -1 (two buffers: fixed)
+    if constexpr (!IP) {
+        xo[0] = x;
+        xo[1] = x > 0 ? x - 1 : nx - 1;
+        xo[2] = x < nx - 1 ? x + 1 : 0;
+        yo[0] = y * nx;
+        yo[1] = (y > 0 ? y - 1 : ny - 1) * nx;
+        yo[2] = (y < ny - 1 ? y + 1 : 0) * nx;
+    }
+    for (int z = zb; z < ze; z += 2) {
+        const int r = ((z - zb) >> 1) & 1;
+        const int s0 = slit_of(P, z), s1 = z + 1 < ze ? slit_of(P, z + 1) : -1;
+        const bool on0 = s0 >= 0 && !frozen(P, s0), on1 = s1 >= 0 && !frozen(P, s1);
+        const bool act0 = in_xy && on0, act1 = in_xy && on1;
+        // both nodes step and none of their sources lies beyond a wall (the
+        // same for the whole CTA)
+        bool both = on0 && on1 && s0 == s1;
+        bool wrap = false;
+        if (both) {
+            const bool inner = z > P.sl[s0].zlo && z + 1 < P.sl[s0].zhi;
+            both = inner || g.zper;
+            wrap = !inner;
+        }
+        PairStage a0, a1;
+        stage_load(z + 1, 0, a0);
+        stage_load(z + 1, 1, a1);
+        float2 v[Q];
+        unsigned bb0 = 0, bb1 = 0;
+        int zo[3][2];  // in place: z offsets of the slots, c_z = 0, +1, -1, of both nodes
+        if (both && (IP || !wrap)) {
+            if (in_xy) {
+                if constexpr (IP) {
+                    const IpSlots q0 = ip_slots(P, P.sl[s0], s0, x, y, z), q1 = ip_slots(P, P.sl[s0], s0, x, y, z + 1);
+                    xo[0] = q0.x, xo[1] = q0.xm, xo[2] = q0.xp;
+                    yo[0] = q0.y * nx, yo[1] = q0.ym * nx, yo[2] = q0.yp * nx;
+                    zo[0][0] = (q0.zb + q0.zr) * nxy, zo[1][0] = (q0.zb + q0.zm) * nxy, zo[2][0] = (q0.zb + q0.zp) * nxy;
+                    zo[0][1] = (q1.zb + q1.zr) * nxy, zo[1][1] = (q1.zb + q1.zm) * nxy, zo[2][1] = (q1.zb + q1.zp) * nxy;
+                }
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    const int cx = kCx(i), cy = kCy(i), cz = kCz(i);
+                    const int o = xo[cx > 0 ? 1 : (cx < 0 ? 2 : 0)] + yo[cy > 0 ? 1 : (cy < 0 ? 2 : 0)];
+                    const T* p = static_cast<const T*>(pp.src[i]);
+                    if constexpr (IP) {
+                        const int k = cz > 0 ? 1 : (cz < 0 ? 2 : 0);
+                        v[i].x = ldq<RAW>(p + (unsigned)(o + zo[k][0]));
+                        v[i].y = ldq<RAW>(p + (unsigned)(o + zo[k][1]));
+                    } else {
+                        v[i].x = ldq<RAW>(p + (unsigned)(o + z * nxy));
+                        v[i].y = ldq<RAW>(p + (unsigned)(o + (z + 1) * nxy));
+                    }
+                }
+            }
+        } else {
+            // the general gathers, one node after the other
+            const T* pin = static_cast<const T*>(pp.src[0]);
+            float w[Q];
+            IpSlots q;
+            if (act0) {
+                if constexpr (IP) q = ip_slots(P, P.sl[s0], s0, x, y, z);
+                csm_pull<0, Q, IP, T, RAW>(P, pin, (long long)z * nxy + y * nx + x, x, y, z, P.sl[s0].zlo, P.sl[s0].zhi,
+                                           w, bb0, q);
+#pragma unroll
+                for (int i = 0; i < Q; ++i) v[i].x = w[i];
+            }
+            if (act1) {
+                if constexpr (IP) q = ip_slots(P, P.sl[s1], s1, x, y, z + 1);
+                csm_pull<0, Q, IP, T, RAW>(P, pin, (long long)(z + 1) * nxy + y * nx + x, x, y, z + 1, P.sl[s1].zlo,
+                                           P.sl[s1].zhi, w, bb1, q);
+#pragma unroll
+                for (int i = 0; i < Q; ++i) v[i].y = w[i];
+            }
+        }
+        __syncthreads();  // the previous round's pairs are read
+        stage_store(z + 1, 0, a0, r ^ 1, r);
+        stage_store(z + 1, 1, a1, r ^ 1, r);
+        __syncthreads();
+        const float2* lo = AB + r * AB_NF * CSM_HN + hc;
+        const float2* hi = AB + (r ^ 1) * AB_NF * CSM_HN + hc;
+        const float2* ow = OW + r * OW_NF * CSM_HN + hc;
+        if (both) {
+            if (!in_xy) continue;
+            if constexpr (RAW) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) v[i] = make_float2(late_cvt(v[i].x), late_cvt(v[i].y));
+            }
+            const float2 dnr = make_float2(lo[AB_DN * CSM_HN].y, hi[AB_DN * CSM_HN].x);
+            auto src = [&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                constexpr int o = -kCx(i) - kCy(i) * CSM_HX, cz = kCz(i);
+                if constexpr (cz != 0)
+                    return SideSrc{(cz > 0 ? lo : hi) + o};
+                else
+                    return LevelSrc{ow + o, lo + o, hi + o};
+            };
+            float2 d79, ux, uy, uz;
+            pull_gather_impl<false>(src, LevelSrc{ow, lo, hi}, (1.f - P.sl[s0].inv_tau) / store_scale<T>(), dnr, 0u, v,
+                                    d79);
+            const int o0 = z * nxy + y * nx + x;
+            auto put = [&](int i, float2 h) {
+                T* p = static_cast<T*>(pp.dst[i]);
+                if constexpr (IP) {
+                    const int cx = kCx(i), cy = kCy(i), cz = kCz(i);
+                    const int o = xo[cx > 0 ? 1 : (cx < 0 ? 2 : 0)] + yo[cy > 0 ? 1 : (cy < 0 ? 2 : 0)];
+                    const int k = cz > 0 ? 1 : (cz < 0 ? 2 : 0);
+                    stp(p + (unsigned)(o + zo[k][0]), h.x);
+                    stp(p + (unsigned)(o + zo[k][1]), h.y);
+                } else {
+                    stp(p + (unsigned)o0, h.x);
+                    stp(p + (unsigned)(o0 + nxy), h.y);
+                }
+            };
+            const float2 dn = pull_finish<T>(put, v, d79, dnr, ux, uy, uz);
+            put_fields(P, io, x, y, z, dn.x, ux.x, uy.x, uz.x, status);
+            put_fields(P, io, x, y, z + 1, dn.y, ux.y, uy.y, uz.y, status);
+            continue;
+        }
+#pragma unroll 1
+        for (int j = 0; j < 2; ++j) {
+            if (!(j ? act1 : act0)) continue;
+            float w[Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                w[i] = j ? v[i].y : v[i].x;
+                if constexpr (RAW) w[i] = late_cvt(w[i]);
+            }
+            const float* fl = reinterpret_cast<const float*>(lo);
+            const float* fh = reinterpret_cast<const float*>(hi);
+            const float* fo = reinterpret_cast<const float*>(ow) + j;
+            const float* own = j ? fh : fl + 1;
+            const float* below = fl + j;
+            const float* above = fh + j;
+            auto src = [&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                constexpr int o = 2 * (-kCx(i) - kCy(i) * CSM_HX), cz = kCz(i);
+                return LoneSrc{fo + o, own + o, (cz > 0 ? below : (cz < 0 ? above : own)) + o};
+            };
+            const int s = j ? s1 : s0;
+            const float dnr = own[2 * AB_DN * CSM_HN];
+            float d79, ux, uy, uz;
+            pull_gather_impl<true>(src, LoneSrc{fo, own, own}, (1.f - P.sl[s].inv_tau) / store_scale<T>(), dnr,
+                                   j ? bb1 : bb0, w, d79);
+            IpSlots q;
+            if constexpr (IP) q = ip_slots(P, P.sl[s], s, x, y, z + j);
+            const int o0 = (z + j) * nxy + y * nx + x;
+            const float dn = pull_finish<T>(
+                [&](int i, float h) { stp(static_cast<T*>(pp.dst[i]) + (unsigned)(IP ? q.slot(i) : o0), h); }, w, d79,
+                dnr, ux, uy, uz);
+            put_fields(P, io, x, y, z + j, dn, ux, uy, uz, status);
+        }
     }
 }
 
@@ -730,10 +1103,25 @@ __global__ void __launch_bounds__(CSM_THREADS, 4)
         csm_collide(own, sm + csm_slot(z - 1) * CSM_SLOT, sm + csm_slot(z + 1) * CSM_SLOT, hc,
                     (1.f - om) / store_scale<T>(), dnr, bb, v, d79);
         float ux, uy, uz;
-        const float dn = pull_finish<T>([&](int i) { return pop_at(pout, P, i, idx); }, v, d79, dnr, ux, uy, uz);
+        const float dn =
+            pull_finish<T>([&](int i, float h) { stp(pop_at(pout, P, i, idx), h); }, v, d79, dnr, ux, uy, uz);
         put_fields(P, io, x, y, z, dn, ux, uy, uz, status);
     }
 }
+
+// a node's staged quantities in registers
+struct Terms {
+    float q[CSM_NF];
+    template <int K>
+    __device__ __forceinline__ float get() const
+    {
+        return q[K];
+    }
+    __device__ __forceinline__ float c0() const
+    {
+        return rest_term(q[SQ_CA], q[SQ_CA + 1], q[SQ_CA + 2], q[SQ_CP], q[SQ_CP + 1], q[SQ_CP + 2]);
+    }
+};
 
 // Narrow grids (below one 32 x 4 tile): the same pass with one thread per
 // node and no staging; every source's quantities are formed where they are
@@ -759,72 +1147,95 @@ __global__ void __launch_bounds__(128) k_pull_node(Params P, const T* pin, T* po
     if constexpr (IP) q = ip_slots(P, P.sl[s], s, x, y, z);
     csm_pull<0, Q, IP>(P, pin, idx, x, y, z, zlo, zhi, v, bb, q);
     const int p = pidx(g, x, y, z);
-    float own[CSM_NF];
-    src_terms(__ldg(io.dn + p), __ldg(io.ux + p), __ldg(io.uy + p), __ldg(io.uz + p), __ldg(F + idx), om, shifted,
-              [&](int j, float val) { own[j] = val; });
-    const float dnr = own[SQ_DN];
+    auto terms_at = [&](int ps, long long nf) {
+        Terms t;
+        const float4 f = __ldg(F + nf);
+        src_terms(__ldg(io.dn + ps), __ldg(io.ux + ps), __ldg(io.uy + ps), __ldg(io.uz + ps), f.x, f.y, f.z, f.w, om,
+                  shifted, [&](int j, float val) { t.q[j] = val; });
+        return t;
+    };
+    const Terms own = terms_at(p, idx);
+    const float dnr = own.q[SQ_DN];
     // the source quantities of direction i, formed where they are used
     // (padded fields through their periodic images, the force at its
     // wrapped node); walls never ask (they use own)
-    auto terms = [&](auto ic, float* out) {
+    auto src = [&](auto ic) {
         constexpr int i = decltype(ic)::value;
         int sx = x - kCx(i), sy = y - kCy(i), sz = z - kCz(i);
         sx = sx < 0 ? sx + g.nx : (sx >= g.nx ? sx - g.nx : sx);
         sy = sy < 0 ? sy + g.ny : (sy >= g.ny ? sy - g.ny : sy);
         if (g.zper) sz = sz < 0 ? sz + g.nz : (sz >= g.nz ? sz - g.nz : sz);
-        const int ps = p - P.nbr[i];
-        src_terms(__ldg(io.dn + ps), __ldg(io.ux + ps), __ldg(io.uy + ps), __ldg(io.uz + ps),
-                  __ldg(F + (((long long)sz * g.ny + sy) * g.nx + sx)), om, shifted,
-                  [&](int j, float val) { out[j] = val; });
+        return terms_at(p - P.nbr[i], ((long long)sz * g.ny + sy) * g.nx + sx);
     };
-    auto wall = [&](int i) { return ((bb >> i) & 1u) != 0u; };
-    auto diff = [&](auto ic, auto ipc) {
-        constexpr int i = decltype(ic)::value, ip = decltype(ipc)::value;
-        if (wall(i)) return mirror_diff<i, ip, 1>(own, own, v[i], v[ip], om1s, true);
-        float a[CSM_NF], b[CSM_NF];
-        terms(ic, a);
-        terms(ipc, b);
-        return mirror_diff<i, ip, 1>(a, b, v[i], v[ip], om1s, false);
-    };
-    using std::integral_constant;
-    const float d7_10 = diff(integral_constant<int, 7>{}, integral_constant<int, 10>{});
-    const float d9_8 = diff(integral_constant<int, 9>{}, integral_constant<int, 8>{});
-    const float d10_8 = diff(integral_constant<int, 10>{}, integral_constant<int, 8>{});
-    const float d79 = diff(integral_constant<int, 7>{}, integral_constant<int, 9>{});
-    v[7] = d7_10;
-    v[9] = d9_8;
-    v[10] = d10_8;
-    v[1] = diff(integral_constant<int, 1>{}, integral_constant<int, 2>{});
-    v[3] = diff(integral_constant<int, 3>{}, integral_constant<int, 4>{});
-    v[11] = diff(integral_constant<int, 11>{}, integral_constant<int, 14>{});
-    v[13] = diff(integral_constant<int, 13>{}, integral_constant<int, 12>{});
-    v[15] = diff(integral_constant<int, 15>{}, integral_constant<int, 18>{});
-    v[17] = diff(integral_constant<int, 17>{}, integral_constant<int, 16>{});
-    auto one = [&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        if constexpr (i == 0 || i == 2 || i == 4 || i == 5 || i == 6 || i == 8 || i == 12 || i == 14 || i == 16 ||
-                      i == 18) {
-            const bool w = i != 0 && wall(i);
-            if (i == 0 || w) {
-                v[i] = arrive<i, 1>(own, v[i], om1s, dnr, w);
-            } else {
-                float sv[CSM_NF];
-                terms(ic, sv);
-                v[i] = arrive<i, 1>(sv, v[i], om1s, dnr, false);
-            }
-        }
-    };
-    for_dirs(one);
+    float d79;
+    pull_gather_impl<true>(src, own, om1s, dnr, bb, v, d79);
     float ux, uy, uz;
-    const float dn = IP ? pull_finish<T>([&](int i) { return pop_at_ip(pout, P, i, q.slot(i)); }, v, d79, dnr, ux,
-                                         uy, uz)
-                        : pull_finish<T>([&](int i) { return pop_at(pout, P, i, idx); }, v, d79, dnr, ux, uy, uz);
+    const float dn =
+        pull_finish<T>([&](int i, float h) { stp(IP ? pop_at_ip(pout, P, i, q.slot(i)) : pop_at(pout, P, i, idx), h); },
+                       v, d79, dnr, ux, uy, uz);
     put_fields(P, io, x, y, z, dn, ux, uy, uz, status);
 }
 
 bool csm_ok(const Geom& g) { return g.nx >= CSM_TX && g.ny >= CSM_TY; }
 
-template <typename T, bool PF, bool IP>
+// z planes per segment when the caller leaves them to the library: the even
+// length that minimises (waves of the NUM_SMS PAIR_MINB resident CTAs) x
+// (planes + 3), the 3 standing for a segment's first two staged planes and its
+// start. Large grids get 32 (512 x 512 x 192: 8 / 16 / 32 / 64 planes 2.27 /
+// 2.20 / 2.19 / 2.23 ms), small ones shorter segments so that every SM has
+// work (64 x 64 x 128: 4 / 8 / 16 / 32 planes 42 / 40 / 53 / 81 us). Many
+// waves overlap, so above four their count is not rounded up.
+static int pair_segment(long long tiles, int nz)
+{
+    int best = 2;
+    double cost = 1e300;
+    for (int lz : {2, 4, 6, 8, 12, 16, 24, 32}) {
+        const double w = (double)(tiles * ((nz + lz - 1) / lz)) / (NUM_SMS * PAIR_MINB);
+        const double c = (w <= 4.0 ? ceil(w) : w) * (lz + 3);
+        if (c <= cost) {
+            cost = c;
+            best = lz;
+        }
+    }
+    return best;
+}
+
+template <typename T, bool IP>
+static cudaError_t pull_pair(const Params& P, const void* pin, void* pout, const CsmIO& io, const float4* F,
+                             int* status, int lz, cudaStream_t s)
+{
+    const Geom& g = P.g;
+    const int tx = (g.nx + CSM_TX - 1) / CSM_TX, ty = (g.ny + CSM_TY - 1) / CSM_TY;
+    if (lz <= 0) lz = pair_segment((long long)tx * ty, g.nz);
+    lz += lz & 1;  // two planes per round
+    const int segs = (g.nz + lz - 1) / lz;
+    const long long blocks = (long long)tx * ty * segs;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const size_t smem = sizeof(float) * PAIR_FLOATS;
+    // the shared-memory limit is a per-device function attribute
+    static std::atomic<uint64_t> configured{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = 1ull << (dev & 63);
+    if (!(configured.load() & bit)) {
+        e = cudaFuncSetAttribute(k_pull_pair<T, IP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        configured.fetch_or(bit);
+    }
+    PullPtrs pp;
+    for (int i = 0; i < Q; ++i) {
+        const int cz = i == 5 || i == 11 || i == 14 || i == 15 || i == 18 ? 1
+                       : (i == 6 || i == 12 || i == 13 || i == 16 || i == 17 ? -1 : 0);
+        const long long back = IP ? 0 : -(long long)cz * g.nx * g.ny;
+        pp.src[i] = static_cast<const T*>(pin) + P.dbase[i] + back;
+        pp.dst[i] = static_cast<T*>(pout) + P.dbase[i];
+    }
+    k_pull_pair<T, IP><<<(unsigned)blocks, CSM_THREADS, smem, s>>>(P, pp, io, F, lz, tx, ty, status);
+    return cudaGetLastError();
+}
+
+template <typename T, bool IP>
 static cudaError_t csm_tiled(const Params& P, const void* pin, void* pout, const CsmIO& io, const float4* F,
                              int* status, int lz, cudaStream_t s)
 {
@@ -841,11 +1252,11 @@ static cudaError_t csm_tiled(const Params& P, const void* pin, void* pout, const
     if (e != cudaSuccess) return e;
     const uint64_t bit = 1ull << (dev & 63);
     if (!(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(k_csm<T, PF, IP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k_csm<T, IP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         configured.fetch_or(bit);
     }
-    k_csm<T, PF, IP><<<(unsigned)blocks, CSM_THREADS, smem, s>>>(P, (const T*)pin, (T*)pout, io, F, lz, tx, ty, status);
+    k_csm<T, IP><<<(unsigned)blocks, CSM_THREADS, smem, s>>>(P, (const T*)pin, (T*)pout, io, F, lz, tx, ty, status);
     return cudaGetLastError();
 }
 
@@ -892,19 +1303,19 @@ cudaError_t launch_csm(const Params& P, const void* pin, void* pout, const CsmIO
         if (!h16 && !ip) k_pull_node<float, false><<<nb, 128, 0, s>>>(P, (const float*)pin, (float*)pout, io, F, status);
         return cudaGetLastError();
     }
-    if (lz <= 0) lz = CSM_LZ;
-    if (h16) {
-        if (ip)
-            return prefetch ? csm_tiled<__half, true, true>(P, pin, pout, io, F, status, lz, s)
-                            : csm_tiled<__half, false, true>(P, pin, pout, io, F, status, lz, s);
-        return prefetch ? csm_tiled<__half, true, false>(P, pin, pout, io, F, status, lz, s)
-                        : csm_tiled<__half, false, false>(P, pin, pout, io, F, status, lz, s);
+    if (prefetch != 1) {
+        if (h16)
+            return ip ? pull_pair<__half, true>(P, pin, pout, io, F, status, lz, s)
+                      : pull_pair<__half, false>(P, pin, pout, io, F, status, lz, s);
+        return ip ? pull_pair<float, true>(P, pin, pout, io, F, status, lz, s)
+                  : pull_pair<float, false>(P, pin, pout, io, F, status, lz, s);
     }
-    if (ip)
-        return prefetch ? csm_tiled<float, true, true>(P, pin, pout, io, F, status, lz, s)
-                        : csm_tiled<float, false, true>(P, pin, pout, io, F, status, lz, s);
-    return prefetch ? csm_tiled<float, true, false>(P, pin, pout, io, F, status, lz, s)
-                    : csm_tiled<float, false, false>(P, pin, pout, io, F, status, lz, s);
+    if (lz <= 0) lz = CSM_LZ;
+    if (h16)
+        return ip ? csm_tiled<__half, true>(P, pin, pout, io, F, status, lz, s)
+                  : csm_tiled<__half, false>(P, pin, pout, io, F, status, lz, s);
+    return ip ? csm_tiled<float, true>(P, pin, pout, io, F, status, lz, s)
+              : csm_tiled<float, false>(P, pin, pout, io, F, status, lz, s);
 }
 
 }  // namespace lbif
