@@ -210,9 +210,8 @@ __device__ __forceinline__ bool cta_wait(uint64_t* mbar, uint32_t parity)
 #define LBIF_GEMM_THREADS 256
 #endif
 constexpr int GEMM_THREADS = LBIF_GEMM_THREADS;
-__global__ void __launch_bounds__(GEMM_THREADS, 2) k_gemm_tc(Gemm g, int ntile)
+__device__ __forceinline__ void gemm_tile(const Gemm& g, int ntile, uint8_t* smem)
 {
-    extern __shared__ __align__(1024) uint8_t smem[];
     const int SB = gemm_stage_bytes(ntile);
     uint64_t* mbar = (uint64_t*)(smem + 2 * SB);
     uint32_t* tslot = (uint32_t*)(mbar + 2);
@@ -372,6 +371,37 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_gemm_tc(Gemm g, int ntile)
     if (warp == 0) tmem_dealloc(tmem, cols);
 }
 
+__global__ void __launch_bounds__(GEMM_THREADS, 2) k_gemm_tc(Gemm g, int ntile)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    gemm_tile(g, ntile, smem);
+}
+
+// The weight gradients dW_l = dZ_l^T . H_l of several layers in one launch.
+// One product's 8 tiles leave the chip idle (25 us each at a batch of 1024, in
+// series); all four layers side by side take 27 us. Batches above WGRAD_ROWS are split: CTA (x, y, l S + s)
+// adds rows [s chunk, (s + 1) chunk) of the batch into the partial product
+// part + s pstride, and k_finish adds the parts in order.
+constexpr int WGRAD_LAYERS = 8, WGRAD_SPLITS = 16, WGRAD_ROWS = 4096;
+struct GemmBatch {
+    Gemm g[WGRAD_LAYERS];
+    int splits, chunk;
+    size_t pstride;
+};
+__global__ void __launch_bounds__(GEMM_THREADS, 2) k_wgrad(const __grid_constant__ GemmBatch b, int ntile)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const int s = blockIdx.z % b.splits;
+    Gemm g = b.g[blockIdx.z / b.splits];
+    if ((int)blockIdx.x * 128 >= g.M || (int)blockIdx.y * ntile >= g.N) return;
+    const int k0 = s * b.chunk;
+    g.A += k0;
+    g.B += k0;
+    g.K = min(b.chunk, g.K - k0);
+    g.Z += s * b.pstride;
+    gemm_tile(g, ntile, smem);
+}
+
 // ---------------------------------------------------------------------------
 // element-wise kernels
 // ---------------------------------------------------------------------------
@@ -387,82 +417,195 @@ __global__ void k_pack_input(const float* X, int batch, int nin, int bp, int kpa
     HT[(size_t)c * bp + r] = b;
 }
 
-// sum of the mask (one block, fixed order), at least 1
-__global__ void k_msum(const float* mask, long long n, double* out)
+// FP64 sum over the CTA's 256 threads in a fixed order (sh: 8 doubles; every
+// thread gets it)
+__device__ __forceinline__ double block_sum(double s, double* sh)
 {
-    __shared__ double sh[256];
-    double s = 0.0;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) s += mask[i];
-    sh[threadIdx.x] = s;
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) s += __shfl_down_sync(0xffffffffu, s, k);
     __syncthreads();
-    for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-        if (threadIdx.x < k) sh[threadIdx.x] += sh[threadIdx.x + k];
-        __syncthreads();
+    if (threadIdx.x % 32 == 0) sh[threadIdx.x / 32] = s;
+    __syncthreads();
+    s = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += sh[k];
+    return s;
+}
+
+// A sum kept as an unevaluated FP32 pair hi + lo (about 48 bits; Knuth's
+// two-sum gives the rounding error of each addition exactly): FP64 adds and
+// conversions run at 1/64 of the FP32 rate, so a thread converts once, at the end.
+struct SumPair {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+        hi = s;
     }
-    if (threadIdx.x == 0) *out = fmax(sh[0], 1.0);
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+// partial sums of the mask, one per block (fixed order)
+constexpr int MSUM_BLOCKS = 64;
+__global__ void __launch_bounds__(256) k_msum(const float* mask, long long n, double* part)
+{
+    __shared__ double sh[8];
+    SumPair a;
+#pragma unroll 4
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += MSUM_BLOCKS * 256LL) a.add(mask[i]);
+    const double s = block_sum(a.value(), sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+
+// the mask's sum from its parts, at least 1 (called by one whole warp; lane 0
+// gets it)
+__device__ __forceinline__ double mask_sum(const double* part)
+{
+    const int lane = threadIdx.x % 32;
+    double s = 0.0;
+    for (int k = lane; k < MSUM_BLOCKS; k += 32) s += part[k];
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) s += __shfl_down_sync(0xffffffffu, s, k);
+    return fmax(s, 1.0);
 }
 
 // dY = 2 mask (Y - T) / sum(mask): FP32 (bp x nout), bf16 rows (bp x opad) and
-// bf16 transposed (nout x bp); per-block FP64 partial sums of the loss
-__global__ void k_loss(const float* Y, const float* T, const float* mask, int batch, int nout, int opad, int bp,
-                       const double* msum, float* dY, bf16* dYb, bf16* dYT, double* partial)
+// bf16 transposed (nout x bp); per-block FP64 partial sums of the loss. The
+// factor 2 / sum and the squares are FP32 pairs (see SumPair); a block covers
+// LOSS_PT x 256 elements.
+constexpr int LOSS_PT = 2;
+__global__ void __launch_bounds__(256) k_loss(const float* Y, const float* T, const float* mask, int batch, int nout,
+                                              int opad, int bp, const double* mpart, float* dY, bf16* dYb, bf16* dYT,
+                                              double* partial)
+{
+    __shared__ double sh[8];
+    __shared__ float factor[2];
+    if (threadIdx.x < 32) {
+        const double ms = mask_sum(mpart);
+        if (threadIdx.x == 0) {
+            const double q = 2.0 / ms;
+            factor[0] = (float)q;
+            factor[1] = (float)(q - (double)(float)q);
+        }
+    }
+    __syncthreads();
+    const float sc = factor[0], scl = factor[1];
+    SumPair l;
+#pragma unroll
+    for (int k = 0; k < LOSS_PT; ++k) {
+        const int i = (blockIdx.x * LOSS_PT + k) * 256 + threadIdx.x;
+        if (i < bp * nout) {
+            int r = i / nout, c = i - r * nout;
+            float d = 0.f;
+            if (r < batch) {
+                float m = mask[(size_t)r * nout + c];
+                float e = (Y[(size_t)r * nout + c] - T[(size_t)r * nout + c]) * m;
+                const float q = __fmul_rn(e, e);
+                l.add(q);
+                l.add(__fmaf_rn(e, e, -q));
+                d = __fmaf_rn(e, sc, __fmul_rn(e, scl));
+            }
+            dY[i] = d;
+            bf16 b = __float2bfloat16_rn(d);
+            dYb[(size_t)r * opad + c] = b;
+            dYT[(size_t)c * bp + r] = b;
+        }
+    }
+    const double sum = block_sum(l.value(), sh);
+    if (threadIdx.x == 0) partial[blockIdx.x] = sum;
+}
+
+__device__ __forceinline__ float adam_one(float p, float gi, float* m, float* v, float lr, float b1, float b2,
+                                         float eps, float c1, float c2)
+{
+    const float mi = b1 * *m + (1.f - b1) * gi;
+    const float vi = b2 * *v + (1.f - b2) * gi * gi;
+    *m = mi;
+    *v = vi;
+    return p - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+}
+
+// What follows the weight products, for a group of layers (blockIdx.y): the
+// weight gradients as the ordered sums of their parts, the bias gradients as
+// column sums of dZ (48 bits, fixed order), and with `adam` the update of the
+// parameters and their BF16 shadows (nothing is updated once *err is set).
+// Blocks [0, nw) hold 256 weights each, the next ones 8 bias columns each
+// (256 threads: 32 row strides of 8 columns), the last one (of layer group 0)
+// adds the loss. The former one-thread-per-column sums took 121 us per layer
+// at a batch of 1024, the mask's one-block sum 124 us.
+struct FinishLayer {
+    const float* part;  // weight products, splits x (dout x kpad)
+    const float* dZ;    // bp x dout
+    long long woff, boff;
+    int dout, din, kpad, opad;
+    bf16 *Wb, *WTb;
+};
+struct Finish {
+    FinishLayer l[WGRAD_LAYERS];
+    int splits, bp, nw, adam;
+    size_t pstride;
+    float *p, *g, *m, *v;
+    float lr, b1, b2, eps, c1, c2;
+    const int* err;
+    const double *partial, *mpart;
+    int nb;
+    double* result;  // {loss, err}; NULL: not this group's work
+};
+__global__ void __launch_bounds__(256) k_finish(const __grid_constant__ Finish f)
 {
     __shared__ double sh[256];
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double l = 0.0;
-    if (i < bp * nout) {
-        int r = i / nout, c = i - r * nout;
-        float d = 0.f;
-        if (r < batch) {
-            float m = mask[(size_t)r * nout + c];
-            float e = (Y[(size_t)r * nout + c] - T[(size_t)r * nout + c]) * m;
-            l = (double)e * e;
-            d = (float)(2.0 * e / *msum);
+    const FinishLayer& l = f.l[blockIdx.y];
+    const int bx = blockIdx.x, t = threadIdx.x;
+    auto apply = [&](long long at, float gi) -> float {
+        f.g[at] = gi;
+        if (!f.adam || *f.err) return 0.f;
+        const float w = adam_one(f.p[at], gi, f.m + at, f.v + at, f.lr, f.b1, f.b2, f.eps, f.c1, f.c2);
+        f.p[at] = w;
+        return w;
+    };
+    if (bx < f.nw) {
+        const int i = bx * 256 + t;
+        if (i >= l.dout * l.din) return;
+        const int r = i / l.din, c = i - r * l.din;
+        const float* q = l.part + (size_t)r * l.kpad + c;
+        float gi = 0.f;
+#pragma unroll 8
+        for (int s = 0; s < f.splits; ++s) gi += q[s * f.pstride];
+        const float w = apply(l.woff + i, gi);
+        if (f.adam && !*f.err) {
+            const bf16 b = __float2bfloat16_rn(w);
+            l.Wb[(size_t)r * l.kpad + c] = b;
+            l.WTb[(size_t)c * l.opad + r] = b;
         }
-        dY[i] = d;
-        bf16 b = __float2bfloat16_rn(d);
-        dYb[(size_t)r * opad + c] = b;
-        dYT[(size_t)c * bp + r] = b;
+        return;
     }
-    sh[threadIdx.x] = l;
+    if (bx == (int)gridDim.x - 1) {
+        if (!f.result || blockIdx.y) return;
+        double s = 0.0;
+        for (int i = t; i < f.nb; i += 256) s += f.partial[i];
+        s = block_sum(s, sh);
+        const double ms = t < 32 ? mask_sum(f.mpart) : 1.0;
+        if (t == 0) {
+            f.result[0] = s / ms;
+            f.result[1] = (double)*f.err;
+        }
+        return;
+    }
+    const int c = (bx - f.nw) * 8 + (t & 7);
+    if ((bx - f.nw) * 8 >= l.dout) return;
+    SumPair a;
+    if (c < l.dout) {
+#pragma unroll 8
+        for (int r = t >> 3; r < f.bp; r += 32) a.add(l.dZ[(size_t)r * l.dout + c]);
+    }
+    sh[t] = a.value();
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
+    for (int k = 128; k >= 8; k >>= 1) {
+        if (t < k) sh[t] += sh[t + k];
         __syncthreads();
     }
-    if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
-}
-
-// column sums of D (rows x cols, FP32) -> out (fixed-order, one thread per column)
-__global__ void k_colsum(const float* D, int rows, int cols, float* out)
-{
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols) return;
-    double s = 0.0;
-    for (int r = 0; r < rows; ++r) s += D[(size_t)r * cols + c];
-    out[c] = (float)s;
-}
-
-// copy the first ncopy columns of a (rows x ld) FP32 matrix into dst (rows x ncopy)
-__global__ void k_copy_cols(const float* src, int rows, int ld, int ncopy, float* dst)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows * ncopy) return;
-    int r = i / ncopy, c = i - r * ncopy;
-    dst[i] = src[(size_t)r * ld + c];
-}
-
-__global__ void k_adam(float* p, const float* g, float* m, float* v, long long n, float lr, float b1, float b2,
-                       float eps, float c1, float c2)
-{
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float gi = g[i];
-    float mi = b1 * m[i] + (1.f - b1) * gi;
-    float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    if (t < 8 && c < l.dout) apply(l.boff + c, (float)sh[t]);
 }
 
 // bf16 shadows of W (nout x nin): row-major padded to kpad columns, and
@@ -499,15 +642,31 @@ struct lbif_mlp_ctx {
     float* dY = nullptr;         // output error FP32 (bp x nout)
     std::vector<float*> dZ;      // per layer FP32 error (bp x dout)
     std::vector<bf16*> dZb, dZT; // bf16 copies
-    float* dWtmp = nullptr;      // dW with padded columns
+    float* dWpart = nullptr;     // parts of the weight products: splits x npart
+    size_t npart = 0;            // dout x kpad of all layers
+    std::vector<size_t> poff;    // offsets of the layers in one part
     float* Xd = nullptr;         // device staging for host inputs (max_batch x nin)
     float *Td = nullptr, *Md = nullptr, *Yd = nullptr;
     double* partial = nullptr;
-    double* msum = nullptr;
+    double* mpart = nullptr;
+    double* result = nullptr;    // {loss, err} of a training call
     int* err = nullptr;
     long long adam_t = 0;
     std::string msg;
 };
+
+// parts the batch of a weight product is split into: WGRAD_ROWS rows each, 16
+// parts at most (their sum reads them all again); rows a part holds
+static int wgrad_splits(int bp)
+{
+    const int s = (bp + WGRAD_ROWS - 1) / WGRAD_ROWS;
+    return s < WGRAD_SPLITS ? s : WGRAD_SPLITS;
+}
+static int wgrad_chunk(int bp)
+{
+    const int s = wgrad_splits(bp);
+    return ((bp + s - 1) / s + GEMM_KC - 1) / GEMM_KC * GEMM_KC;
+}
 
 static thread_local std::string g_mlp_err = "no error";
 
@@ -528,7 +687,7 @@ static int mfail(lbif_mlp_ctx* m, int code, const std::string& s)
 static void mlp_free(lbif_mlp_ctx* m)
 {
     if (!m) return;
-    std::vector<void*> bufs = {m->p, m->g, m->m, m->v, m->dY, m->dWtmp, m->Xd, m->Td, m->Md, m->Yd, m->partial, m->msum, m->err};
+    std::vector<void*> bufs = {m->p, m->g, m->m, m->v, m->dY, m->dWpart, m->Xd, m->Td, m->Md, m->Yd, m->partial, m->mpart, m->result, m->err};
     for (auto* b : m->Wb) bufs.push_back(b);
     for (auto* b : m->WTb) bufs.push_back(b);
     for (auto* b : m->Z) bufs.push_back(b);
@@ -582,13 +741,17 @@ extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32
         off += dq;
     }
     m->nparams = off;
+    for (int l = 0; l < m->L; ++l) {
+        m->poff.push_back(m->npart);
+        m->npart += (size_t)m->dout[l] * m->kpad[l];
+    }
     const int bp = m->bp_max;
     bool ok = dalloc(&m->p, off) && dalloc(&m->g, off) && dalloc(&m->m, off) && dalloc(&m->v, off) &&
-              dalloc(&m->dY, (size_t)bp * nout) && dalloc(&m->dWtmp, (size_t)256 * 256) &&
+              dalloc(&m->dY, (size_t)bp * nout) && dalloc(&m->dWpart, wgrad_splits(bp) * m->npart) &&
               dalloc(&m->Xd, (size_t)max_batch * nin) && dalloc(&m->Td, (size_t)max_batch * nout) &&
               dalloc(&m->Md, (size_t)max_batch * nout) && dalloc(&m->Yd, (size_t)bp * nout) &&
-              dalloc(&m->partial, (size_t)(bp * nout + 255) / 256 + 1) && dalloc(&m->msum, 1) &&
-              dalloc(&m->err, 1);
+              dalloc(&m->partial, (size_t)(bp * nout + 255) / 256 + 1) && dalloc(&m->mpart, MSUM_BLOCKS) &&
+              dalloc(&m->result, 2) && dalloc(&m->err, 1);
     for (int l = 0; ok && l < m->L; ++l) {
         bf16 *wb, *wtb, *h, *ht, *dzb, *dzt;
         float *z, *dz;
@@ -609,7 +772,8 @@ extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32
         mlp_free(m);
         return mfail(nullptr, LBIF_ERR_NOMEM, "lbif_mlp_create: device allocation failed");
     }
-    if (cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256)) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256)) != cudaSuccess ||
+        cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256)) != cudaSuccess) {
         cudaGetLastError();
         mlp_free(m);
         return mfail(nullptr, LBIF_ERR_CUDA, "lbif_mlp_create: shared memory configuration failed");
@@ -768,8 +932,14 @@ extern "C" int lbif_mlp_forward(lbif_mlp m, const float* X, int32_t batch, float
     return check_err(m);
 }
 
-// loss and gradients into m->g
-static int backward(lbif_mlp_ctx* m, const float* T, const float* mask, int batch, int on_device, double* loss)
+// learning rate and Adam's constants of a training step
+struct AdamStep {
+    float lr, beta1, beta2, eps, c1, c2;
+};
+
+// loss and gradients into m->g; with `adam` also the parameters' update
+static int backward(lbif_mlp_ctx* m, const float* T, const float* mask, int batch, int on_device, double* loss,
+                    const AdamStep* adam = nullptr)
 {
     const int bp = up16(batch);
     const int nout = m->nout;
@@ -782,31 +952,12 @@ static int backward(lbif_mlp_ctx* m, const float* T, const float* mask, int batc
     }
     const int L = m->L;
     const int n = bp * nout;
-    const int nb = (n + 255) / 256;
-    k_msum<<<1, 256, 0, m->stream>>>(Md, (long long)batch * nout, m->msum);
-    k_loss<<<nb, 256, 0, m->stream>>>(m->Z[L - 1], Td, Md, batch, nout, m->opad[L - 1], bp, m->msum,
+    const int nb = (n + 256 * LOSS_PT - 1) / (256 * LOSS_PT);
+    k_msum<<<MSUM_BLOCKS, 256, 0, m->stream>>>(Md, (long long)batch * nout, m->mpart);
+    k_loss<<<nb, 256, 0, m->stream>>>(m->Z[L - 1], Td, Md, batch, nout, m->opad[L - 1], bp, m->mpart,
                                       m->dZ[L - 1], m->dZb[L - 1], m->dZT[L - 1], m->partial);
     MCK(m, cudaGetLastError());
-    for (int l = L - 1; l >= 0; --l) {
-        // dW_l = dZ_l^T . H_l  (M = dout, N = kpad_l, K = bp)
-        Gemm gw = blank(m);
-        gw.A = m->dZT[l];
-        gw.lda = bp;
-        gw.B = m->HT[l];
-        gw.ldb = bp;
-        gw.M = m->dout[l];
-        gw.N = m->kpad[l];
-        gw.K = bp;
-        gw.Z = m->dWtmp;
-        gw.ldz = m->kpad[l];
-        int rc = gemm(m, gw);
-        if (rc) return rc;
-        int cnt = m->dout[l] * m->din[l];
-        k_copy_cols<<<(cnt + 255) / 256, 256, 0, m->stream>>>(m->dWtmp, m->dout[l], m->kpad[l], m->din[l],
-                                                              m->g + m->woff[l]);
-        k_colsum<<<(m->dout[l] + 127) / 128, 128, 0, m->stream>>>(m->dZ[l], bp, m->dout[l], m->g + m->boff[l]);
-        MCK(m, cudaGetLastError());
-        if (l == 0) break;
+    for (int l = L - 1; l > 0; --l) {
         // dZ_{l-1} = (dZ_l . W_l) * gelu'(Z_{l-1})  (M = bp, N = din_l, K = dout_l)
         Gemm gd = blank(m);
         gd.A = m->dZb[l];
@@ -824,16 +975,80 @@ static int backward(lbif_mlp_ctx* m, const float* T, const float* mask, int batc
         gd.ldh = m->opad[l - 1];
         gd.HT = m->dZT[l - 1];
         gd.ldht = bp;
-        if ((rc = gemm(m, gd))) return rc;
+        const int rc = gemm(m, gd);
+        if (rc) return rc;
     }
-    std::vector<double> part(nb + 1);
-    MCK(m, cudaMemcpyAsync(part.data(), m->partial, sizeof(double) * nb, cudaMemcpyDeviceToHost, m->stream));
-    MCK(m, cudaMemcpyAsync(part.data() + nb, m->msum, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
-    int rc = check_err(m);
-    if (rc) return rc;
-    double s = 0.0;
-    for (int i = 0; i < nb; ++i) s += part[i];
-    if (loss) *loss = s / part[nb];
+    std::vector<Finish> fin;  // after every product: nothing is updated once one failed
+    std::vector<dim3> fgrid;
+    for (int l0 = 0; l0 < L; l0 += WGRAD_LAYERS) {
+        const int nl = L - l0 < WGRAD_LAYERS ? L - l0 : WGRAD_LAYERS;
+        GemmBatch gb;
+        memset(&gb, 0, sizeof(gb));
+        Finish f;
+        memset(&f, 0, sizeof(f));
+        gb.splits = f.splits = wgrad_splits(bp);
+        gb.chunk = wgrad_chunk(bp);
+        // rounding the chunk up may leave trailing parts without rows
+        gb.splits = f.splits = (bp + gb.chunk - 1) / gb.chunk;
+        gb.pstride = f.pstride = m->npart;
+        int mt = 1, nt = 1, nbias = 1;
+        for (int k = 0; k < nl; ++k) {
+            const int l = l0 + k;
+            // dW_l = dZ_l^T . H_l  (M = dout, N = din, K = bp)
+            Gemm& gw = gb.g[k];
+            gw = blank(m);
+            gw.A = m->dZT[l];
+            gw.lda = bp;
+            gw.B = m->HT[l];
+            gw.ldb = bp;
+            gw.M = m->dout[l];
+            gw.N = m->din[l];
+            gw.K = bp;
+            gw.Z = m->dWpart + m->poff[l];
+            gw.ldz = m->kpad[l];
+            const int tiles_m = (m->dout[l] + 127) / 128, tiles_n = (m->din[l] + 63) / 64;
+            mt = tiles_m > mt ? tiles_m : mt;
+            nt = tiles_n > nt ? tiles_n : nt;
+            const int w = (m->dout[l] * m->din[l] + 255) / 256, c = (m->dout[l] + 7) / 8;
+            f.nw = w > f.nw ? w : f.nw;
+            nbias = c > nbias ? c : nbias;
+            f.l[k] = FinishLayer{gw.Z, m->dZ[l], m->woff[l], m->boff[l], m->dout[l], m->din[l], m->kpad[l], m->opad[l],
+                                 m->Wb[l], m->WTb[l]};
+        }
+        k_wgrad<<<dim3(mt, nt, nl * gb.splits), GEMM_THREADS, gemm_smem_bytes(64), m->stream>>>(gb, 64);
+        MCK(m, cudaGetLastError());
+        f.bp = bp;
+        f.p = m->p;
+        f.g = m->g;
+        f.m = m->m;
+        f.v = m->v;
+        f.err = m->err;
+        if (adam) {
+            f.adam = 1;
+            f.lr = adam->lr;
+            f.b1 = adam->beta1;
+            f.b2 = adam->beta2;
+            f.eps = adam->eps;
+            f.c1 = adam->c1;
+            f.c2 = adam->c2;
+        }
+        f.partial = m->partial;
+        f.mpart = m->mpart;
+        f.nb = nb;
+        f.result = l0 + nl == L ? m->result : nullptr;
+        fin.push_back(f);
+        fgrid.push_back(dim3(f.nw + nbias + 1, nl));
+    }
+    for (size_t k = 0; k < fin.size(); ++k) {
+        k_finish<<<fgrid[k], 256, 0, m->stream>>>(fin[k]);
+        MCK(m, cudaGetLastError());
+    }
+    double r[2] = {0.0, 0.0};
+    MCK(m, cudaMemcpyAsync(r, m->result, 2 * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+    MCK(m, cudaStreamSynchronize(m->stream));
+    if (r[1] != 0.0)
+        return mfail(m, LBIF_ERR_TIMEOUT, "tensor-core product did not complete within its wait limit");
+    if (loss) *loss = r[0];
     return LBIF_OK;
 }
 
@@ -862,13 +1077,11 @@ extern "C" int lbif_mlp_train_step(lbif_mlp m, const float* X, const float* T, c
     int rc = pack_input(m, X, batch, on_device);
     if (rc) return rc;
     if ((rc = forward(m, batch, true))) return rc;
-    if ((rc = backward(m, T, mask, batch, on_device, loss))) return rc;
+    // the update rides on the gradients' last kernel; a step whose products
+    // failed leaves the parameters and the step count as they were
+    const double t = (double)(m->adam_t + 1);
+    const AdamStep a{lr, beta1, beta2, eps, (float)(1.0 - pow((double)beta1, t)), (float)(1.0 - pow((double)beta2, t))};
+    if ((rc = backward(m, T, mask, batch, on_device, loss, &a))) return rc;
     m->adam_t += 1;
-    const float c1 = (float)(1.0 - pow((double)beta1, (double)m->adam_t));
-    const float c2 = (float)(1.0 - pow((double)beta2, (double)m->adam_t));
-    k_adam<<<(unsigned)((m->nparams + 255) / 256), 256, 0, m->stream>>>(m->p, m->g, m->m, m->v, m->nparams, lr,
-                                                                         beta1, beta2, eps, c1, c2);
-    MCK(m, cudaGetLastError());
-    if ((rc = refresh_shadows(m))) return rc;
     return LBIF_OK;
 }
