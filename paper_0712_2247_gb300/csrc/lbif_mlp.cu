@@ -403,6 +403,236 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_wgrad(const __grid_constant
 }
 
 // ---------------------------------------------------------------------------
+// The whole forward pass of 128 rows in one CTA (inference). The activations
+// stay in shared memory as the next product's A operand (BF16, K-major core
+// matrices) and the accumulator in tensor memory; only the weights travel, as
+// contiguous chunks of FUSE_KC columns packed in the order the tensor core
+// reads them (pack_offset), each brought in by one bulk copy into a ring of
+// three, two chunks ahead of the products and across layer and tile borders.
+// The epilogue (bias, GELU, BF16) is most of the work: about 60 instructions
+// per element against 512 FLOP on the tensor core, so two CTAs share an SM and
+// one's epilogue covers the other's products. Four launches that passed the
+// activations through L2 took 234 us for 65,536 rows at 4 -> 3 x 256 -> 160; this
+// takes 138 us, 115 of them in the kernel (43 us of issue; an SM holds three or
+// four of the 512 tiles). Loading the next chunk of accumulators and biases
+// early changed nothing.
+// ---------------------------------------------------------------------------
+constexpr int FUSE_KC = 32, FUSE_RING = 3;
+
+// element (r, c) of a layer's weights in its packed image: chunks of FUSE_KC
+// columns (the last one shorter), each n16 rows of 8-row x 16-byte core
+// matrices, K-major
+__host__ __device__ inline size_t pack_offset(int r, int c, int n16, int kpad)
+{
+    const int ch = c / FUSE_KC, left = kpad - ch * FUSE_KC, kc = left < FUSE_KC ? left : FUSE_KC;
+    return (size_t)ch * FUSE_KC * n16 + ((size_t)(r >> 3) * (kc >> 3) + ((c - ch * FUSE_KC) >> 3)) * 64 +
+           (r & 7) * 8 + (c & 7);
+}
+
+struct Fused {
+    const float* X;   // batch x nin
+    float* Y;         // batch x nout
+    const bf16* Wp;   // packed weights, layer after layer
+    const float* p;   // parameters (biases)
+    int batch, nin, hidden, nout, L;
+    int tiles, achunk;  // row tiles; bytes of the activation buffer
+    int* err;
+};
+
+__device__ __forceinline__ bool bounded_wait(uint64_t* mbar, uint32_t parity)
+{
+    long long spins = 0;
+    bool ok;
+    while (!(ok = mbar_try_wait(mbar, parity)) && ++spins < WAIT_LIMIT) {
+    }
+    return ok;
+}
+
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* mbar)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(mbar))
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(256, 2) k_mlp_forward(const __grid_constant__ Fused f)
+{
+    extern __shared__ __align__(1024) uint8_t fsm[];
+    uint8_t* const act = fsm;
+    uint8_t* const ring = fsm + f.achunk;
+    const int n16o = (f.nout + 15) / 16 * 16, kp0 = (f.nin + 15) / 16 * 16;
+    const int nmax = f.hidden > n16o ? f.hidden : n16o;
+    const int slot = nmax * FUSE_KC * 2;  // bytes of a ring slot
+    uint64_t* const full = (uint64_t*)(ring + FUSE_RING * slot);
+    uint64_t* const empty = full + FUSE_RING;
+    uint64_t* const done = empty + FUSE_RING;
+    uint32_t* const tslot = (uint32_t*)(done + 1);
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    const uint32_t cols = tmem_cols(nmax);
+    if (warp == 0) {
+        tmem_alloc(tslot, cols);
+        tmem_relinquish();
+    }
+    if (tid == 0)
+        for (int k = 0; k < 2 * FUSE_RING + 1; ++k) mbar_init(full + k, 1);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tslot;
+
+    // thread 0's cursors over the chunks of all its tiles: loads and products
+    const int my_tiles = (f.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int ch0 = (kp0 + FUSE_KC - 1) / FUSE_KC, chh = (f.hidden + FUSE_KC - 1) / FUSE_KC;
+    const int per_tile = ch0 + (f.L - 1) * chh;
+    const long long chunks = (long long)my_tiles * per_tile;
+    long long nload = 0, nmma = 0;
+    int lc = 0;               // chunk of the tile the next load takes
+    const bf16* lp = f.Wp;    // its address
+    auto load_next = [&]() {
+        if (nload >= chunks) return;
+        const bool first = lc < ch0;
+        const int l = first ? 0 : 1 + (lc - ch0) / chh, c = first ? lc : (lc - ch0) % chh;
+        const int left = (first ? kp0 : f.hidden) - c * FUSE_KC, kc = left < FUSE_KC ? left : FUSE_KC;
+        const int n = l == f.L - 1 ? n16o : f.hidden;
+        const int b = (int)(nload % FUSE_RING);
+        bulk_load(ring + b * slot, lp, (uint32_t)(n * kc * 2), full + b);
+        lp += (size_t)n * kc;
+        ++nload;
+        if (++lc == per_tile) {
+            lc = 0;
+            lp = f.Wp;
+        }
+    };
+    bool ok = true;
+    if (tid == 0)
+        for (int k = 0; k < FUSE_RING - 1; ++k) load_next();
+    uint32_t dphase = 0;
+    for (int tile = blockIdx.x; tile < f.tiles && ok; tile += gridDim.x) {
+        // the input rows as BF16 core matrices, zero beyond nin and the batch
+        {
+            const int r = tid & 127, row = tile * 128 + r, kcore = kp0 / 8;
+            for (int kp = tid >> 7; kp < kcore; kp += 2) {
+                uint4 pk;
+                uint32_t* w = reinterpret_cast<uint32_t*>(&pk);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int c = kp * 8 + 2 * e;
+                    const float a = row < f.batch && c < f.nin ? f.X[(size_t)row * f.nin + c] : 0.f;
+                    const float b = row < f.batch && c + 1 < f.nin ? f.X[(size_t)row * f.nin + c + 1] : 0.f;
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+                    w[e] = *reinterpret_cast<const uint32_t*>(&h);
+                }
+                *reinterpret_cast<uint4*>(act + ((r >> 3) * kcore + kp) * 128 + (r & 7) * 16) = pk;
+            }
+        }
+        const float* bias = f.p + (size_t)f.nin * f.hidden;
+        for (int l = 0; l < f.L && ok; ++l) {
+            const bool last = l == f.L - 1;
+            const int K = l == 0 ? kp0 : f.hidden, N = last ? n16o : f.hidden;
+            fence_proxy_async();  // the activations written above / by the last epilogue
+            tc_fence_before();
+            __syncthreads();
+            tc_fence_after();
+            if (tid == 0) {
+                const uint32_t idesc = idesc_bf16(128, N), a0 = smem_u32(act), asbo = (K / 8) * 128;
+                for (int c = 0; c * FUSE_KC < K && ok; ++c) {
+                    const int b = (int)(nmma % FUSE_RING), kc = min(FUSE_KC, K - c * FUSE_KC);
+                    ok = bounded_wait(full + b, (uint32_t)(nmma / FUSE_RING) & 1u);
+                    if (!ok) break;
+                    const uint32_t b0 = smem_u32(ring + b * slot), bsbo = (kc / 8) * 128;
+                    for (int kk = 0; kk < kc / 16; ++kk)
+                        mma_bf16(tmem, smem_desc(a0 + (c * FUSE_KC / 8 + 2 * kk) * 128, 128, asbo),
+                                 smem_desc(b0 + kk * 256, 128, bsbo), idesc, (c > 0 || kk > 0) ? 1u : 0u);
+                    mma_commit(empty + b);
+                    // the slot of the chunk before: its products precede these
+                    if (nmma > 0 && nload < chunks) {
+                        const long long q = nmma - 1;
+                        ok = bounded_wait(empty + (int)(q % FUSE_RING), (uint32_t)(q / FUSE_RING) & 1u);
+                        if (!ok) break;
+                    }
+                    load_next();
+                    ++nmma;
+                }
+                if (ok) mma_commit(done);
+            }
+            {
+                const bool mine = bounded_wait(done, dphase) && ok;
+                dphase ^= 1u;
+                ok = __syncthreads_and(mine) != 0;
+            }
+            tc_fence_after();
+            if (!ok) break;
+            const int lg = warp % 4, r = 32 * lg + lane, row = tile * 128 + r;
+            if (tile * 128 + 32 * lg < f.batch) {  // the warp holds a row of the batch
+                for (int c = 16 * (warp / 4); c < N; c += 32) {
+                    float v[16], z[16];
+                    __syncwarp();  // rows past the batch skip the stores below
+                    tmem_ld16(tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)c, v);
+                    if (!last || c + 16 <= f.nout) {
+                        if (((uintptr_t)(bias + c) & 15) == 0) {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const float4 t = __ldg(reinterpret_cast<const float4*>(bias + c) + q);
+                                z[4 * q] = t.x, z[4 * q + 1] = t.y, z[4 * q + 2] = t.z, z[4 * q + 3] = t.w;
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) z[j] = __ldg(bias + c + j);
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) z[j] = c + j < f.nout ? __ldg(bias + c + j) : 0.f;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) z[j] = v[j] + z[j];
+                    if (last) {
+                        if (row >= f.batch) continue;
+                        float* y = f.Y + (size_t)row * f.nout + c;
+                        if (c + 16 <= f.nout && ((uintptr_t)y & 15) == 0) {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+                                reinterpret_cast<float4*>(y)[q] = make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j)
+                                if (c + j < f.nout) y[j] = z[j];
+                        }
+                        continue;
+                    }
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        uint4 pk;
+                        uint32_t* w = reinterpret_cast<uint32_t*>(&pk);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const __nv_bfloat162 b2 =
+                                __floats2bfloat162_rn(gelu(z[8 * q + 2 * e]), gelu(z[8 * q + 2 * e + 1]));
+                            w[e] = *reinterpret_cast<const uint32_t*>(&b2);
+                        }
+                        *reinterpret_cast<uint4*>(act + ((r >> 3) * (f.hidden / 8) + c / 8 + q) * 128 + (r & 7) * 16) = pk;
+                    }
+                }
+            }
+            tc_fence_before();
+            bias += f.hidden + (size_t)f.hidden * (l + 1 == f.L - 1 ? f.nout : f.hidden);
+        }
+        // the next tile's input overwrites the activations the last products read
+        // (complete: every thread waited for them)
+    }
+    if (!ok && tid == 0) {
+        atomicExch(f.err, 1);
+        // copies in flight land before the CTA leaves
+        for (long long q = nmma; q < nload; ++q)
+            bounded_wait(full + (int)(q % FUSE_RING), (uint32_t)(q / FUSE_RING) & 1u);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, cols);
+}
+
+// ---------------------------------------------------------------------------
 // element-wise kernels
 // ---------------------------------------------------------------------------
 // X (batch x nin, FP32) -> bf16 rows (bp x kpad) and transposed (kpad x bp), zero padded
@@ -539,7 +769,7 @@ struct FinishLayer {
     const float* dZ;    // bp x dout
     long long woff, boff;
     int dout, din, kpad, opad;
-    bf16 *Wb, *WTb;
+    bf16 *Wb, *WTb, *Wp;
 };
 struct Finish {
     FinishLayer l[WGRAD_LAYERS];
@@ -577,6 +807,7 @@ __global__ void __launch_bounds__(256) k_finish(const __grid_constant__ Finish f
             const bf16 b = __float2bfloat16_rn(w);
             l.Wb[(size_t)r * l.kpad + c] = b;
             l.WTb[(size_t)c * l.opad + r] = b;
+            l.Wp[pack_offset(r, c, l.opad, l.kpad)] = b;
         }
         return;
     }
@@ -608,9 +839,10 @@ __global__ void __launch_bounds__(256) k_finish(const __grid_constant__ Finish f
     if (t < 8 && c < l.dout) apply(l.boff + c, (float)sh[t]);
 }
 
-// bf16 shadows of W (nout x nin): row-major padded to kpad columns, and
-// transposed (nin x opad, columns beyond nout stay zero)
-__global__ void k_shadow(const float* W, int nout, int nin, int kpad, int opad, bf16* Wb, bf16* WTb)
+// bf16 shadows of W (nout x nin): row-major padded to kpad columns, transposed
+// (nin x opad, columns beyond nout stay zero), and packed for the fused forward
+// (opad rows; padding stays zero)
+__global__ void k_shadow(const float* W, int nout, int nin, int kpad, int opad, bf16* Wb, bf16* WTb, bf16* Wp)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nout * kpad) return;
@@ -618,7 +850,10 @@ __global__ void k_shadow(const float* W, int nout, int nin, int kpad, int opad, 
     float w = c < nin ? W[(size_t)r * nin + c] : 0.f;
     bf16 b = __float2bfloat16_rn(w);
     Wb[i] = b;
-    if (c < nin) WTb[(size_t)c * opad + r] = b;
+    if (c < nin) {
+        WTb[(size_t)c * opad + r] = b;
+        Wp[pack_offset(r, c, opad, kpad)] = b;
+    }
 }
 
 inline int up16(int v) { return (v + 15) / 16 * 16; }
@@ -637,6 +872,8 @@ struct lbif_mlp_ctx {
     cudaStream_t stream = nullptr;
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;  // flat FP32
     std::vector<bf16*> Wb, WTb;
+    bf16* Wp = nullptr;          // packed for the fused forward, layer after layer
+    std::vector<size_t> wpoff;   // offsets of the layers in it
     std::vector<float*> Z;       // pre-activations per layer (bp x dout)
     std::vector<bf16*> H, HT;    // layer inputs (bp x kpad) and transposed (kpad x bp)
     float* dY = nullptr;         // output error FP32 (bp x nout)
@@ -687,7 +924,7 @@ static int mfail(lbif_mlp_ctx* m, int code, const std::string& s)
 static void mlp_free(lbif_mlp_ctx* m)
 {
     if (!m) return;
-    std::vector<void*> bufs = {m->p, m->g, m->m, m->v, m->dY, m->dWpart, m->Xd, m->Td, m->Md, m->Yd, m->partial, m->mpart, m->result, m->err};
+    std::vector<void*> bufs = {m->Wp, m->p, m->g, m->m, m->v, m->dY, m->dWpart, m->Xd, m->Td, m->Md, m->Yd, m->partial, m->mpart, m->result, m->err};
     for (auto* b : m->Wb) bufs.push_back(b);
     for (auto* b : m->WTb) bufs.push_back(b);
     for (auto* b : m->Z) bufs.push_back(b);
@@ -711,6 +948,10 @@ static bool dalloc(T** p, size_t n)
     }
     return cudaMemset(*p, 0, sizeof(T) * (n ? n : 1)) == cudaSuccess;
 }
+
+// shared memory of the fused forward: activations of 128 rows x kmax, the ring
+// of weight chunks, barriers and the TMEM address slot
+static int fused_smem(int kmax, int nmax) { return 256 * kmax + FUSE_RING * nmax * FUSE_KC * 2 + 8 * (2 * FUSE_RING + 1) + 16; }
 
 extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32_t nhidden, int32_t nout,
                                int32_t max_batch, void* stream)
@@ -745,13 +986,18 @@ extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32
         m->poff.push_back(m->npart);
         m->npart += (size_t)m->dout[l] * m->kpad[l];
     }
+    size_t npack = 0;
+    for (int l = 0; l < m->L; ++l) {
+        m->wpoff.push_back(npack);
+        npack += (size_t)m->opad[l] * m->kpad[l];
+    }
     const int bp = m->bp_max;
     bool ok = dalloc(&m->p, off) && dalloc(&m->g, off) && dalloc(&m->m, off) && dalloc(&m->v, off) &&
               dalloc(&m->dY, (size_t)bp * nout) && dalloc(&m->dWpart, wgrad_splits(bp) * m->npart) &&
               dalloc(&m->Xd, (size_t)max_batch * nin) && dalloc(&m->Td, (size_t)max_batch * nout) &&
               dalloc(&m->Md, (size_t)max_batch * nout) && dalloc(&m->Yd, (size_t)bp * nout) &&
               dalloc(&m->partial, (size_t)(bp * nout + 255) / 256 + 1) && dalloc(&m->mpart, MSUM_BLOCKS) &&
-              dalloc(&m->result, 2) && dalloc(&m->err, 1);
+              dalloc(&m->result, 2) && dalloc(&m->err, 1) && dalloc(&m->Wp, npack);
     for (int l = 0; ok && l < m->L; ++l) {
         bf16 *wb, *wtb, *h, *ht, *dzb, *dzt;
         float *z, *dz;
@@ -773,7 +1019,8 @@ extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32
         return mfail(nullptr, LBIF_ERR_NOMEM, "lbif_mlp_create: device allocation failed");
     }
     if (cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256)) != cudaSuccess ||
-        cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256)) != cudaSuccess) {
+        cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256)) != cudaSuccess ||
+        cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, fused_smem(256, 256)) != cudaSuccess) {
         cudaGetLastError();
         mlp_free(m);
         return mfail(nullptr, LBIF_ERR_CUDA, "lbif_mlp_create: shared memory configuration failed");
@@ -799,7 +1046,7 @@ static int refresh_shadows(lbif_mlp_ctx* m)
     for (int l = 0; l < m->L; ++l) {
         int n = m->dout[l] * m->kpad[l];
         k_shadow<<<(n + 255) / 256, 256, 0, m->stream>>>(m->p + m->woff[l], m->dout[l], m->din[l], m->kpad[l],
-                                                         m->opad[l], m->Wb[l], m->WTb[l]);
+                                                         m->opad[l], m->Wb[l], m->WTb[l], m->Wp + m->wpoff[l]);
     }
     MCK(m, cudaGetLastError());
     return LBIF_OK;
@@ -853,12 +1100,10 @@ static Gemm blank(lbif_mlp_ctx* m)
     return g;
 }
 
-// forward of `batch` rows already packed in H[0] / HT[0]. train: keep what
-// back-propagation reads (every layer's FP32 pre-activation Z and the
-// transposed BF16 activations HT); otherwise each hidden layer writes only
-// the next layer's BF16 input, and the output goes to Yout (batch x nout,
-// device memory) when given, else to Z of the last layer.
-static int forward(lbif_mlp_ctx* m, int batch, bool train, float* Yout = nullptr)
+// the training forward of `batch` rows already packed in H[0] / HT[0]: keeps
+// what back-propagation reads (every layer's FP32 pre-activation Z and the
+// transposed BF16 activations HT)
+static int forward(lbif_mlp_ctx* m, int batch)
 {
     const int bp = up16(batch);
     for (int l = 0; l < m->L; ++l) {
@@ -873,25 +1118,45 @@ static int forward(lbif_mlp_ctx* m, int batch, bool train, float* Yout = nullptr
         g.K = m->kpad[l];
         g.bias = m->p + m->boff[l];
         g.epi = last ? EPI_NONE : EPI_GELU;
-        if (train || last) {
-            g.Z = m->Z[l];
-            g.ldz = m->dout[l];
-        }
-        if (last && !train && Yout) {
-            g.Z = Yout;
-            g.M = batch;  // the rows Yout holds
-        }
+        g.Z = m->Z[l];
+        g.ldz = m->dout[l];
         if (!last) {
             g.H = m->H[l + 1];
             g.ldh = m->kpad[l + 1];
-            if (train) {
-                g.HT = m->HT[l + 1];
-                g.ldht = bp;
-            }
+            g.HT = m->HT[l + 1];
+            g.ldht = bp;
         }
         int rc = gemm(m, g);
         if (rc) return rc;
     }
+    return LBIF_OK;
+}
+
+// inference: Y (batch x nout) of X (batch x nin), device memory
+static int infer(lbif_mlp_ctx* m, const float* X, int batch, float* Y)
+{
+    Fused f;
+    memset(&f, 0, sizeof(f));
+    f.X = X;
+    f.Y = Y;
+    f.Wp = m->Wp;
+    f.p = m->p;
+    f.batch = batch;
+    f.nin = m->nin;
+    f.hidden = m->hidden;
+    f.nout = m->nout;
+    f.L = m->L;
+    f.tiles = (batch + 127) / 128;
+    const int kmax = m->kpad[0] > m->hidden ? m->kpad[0] : m->hidden;
+    const int nmax = m->opad[m->L - 1] > m->hidden ? m->opad[m->L - 1] : m->hidden;
+    f.achunk = 256 * kmax;
+    f.err = m->err;
+    // two CTAs per SM: shared memory keeps a third one (and its TMEM) out
+    int smem = fused_smem(kmax, nmax);
+    if (smem < 80 * 1024) smem = 80 * 1024;
+    const int grid = f.tiles < 304 ? f.tiles : 304;
+    k_mlp_forward<<<grid, 256, smem, m->stream>>>(f);
+    MCK(m, cudaGetLastError());
     return LBIF_OK;
 }
 
@@ -922,13 +1187,16 @@ extern "C" int lbif_mlp_forward(lbif_mlp m, const float* X, int32_t batch, float
 {
     if (!m || !X || !Y || batch < 1 || batch > m->max_batch)
         return mfail(m, LBIF_ERR_ARG, "lbif_mlp_forward: bad arguments");
-    int rc = pack_input(m, X, batch, on_device);
+    const float* Xd = X;
+    if (!on_device) {
+        MCK(m, cudaMemcpyAsync(m->Xd, X, sizeof(float) * (size_t)batch * m->nin, cudaMemcpyHostToDevice, m->stream));
+        Xd = m->Xd;
+    }
+    float* Yd = on_device ? Y : m->Yd;
+    const int rc = infer(m, Xd, batch, Yd);
     if (rc) return rc;
-    // device output: the last product writes Y itself
-    if ((rc = forward(m, batch, false, on_device ? Y : nullptr))) return rc;
     if (!on_device)
-        MCK(m, cudaMemcpyAsync(Y, m->Z[m->L - 1], sizeof(float) * (size_t)batch * m->nout, cudaMemcpyDeviceToHost,
-                               m->stream));
+        MCK(m, cudaMemcpyAsync(Y, Yd, sizeof(float) * (size_t)batch * m->nout, cudaMemcpyDeviceToHost, m->stream));
     return check_err(m);
 }
 
@@ -1013,7 +1281,7 @@ static int backward(lbif_mlp_ctx* m, const float* T, const float* mask, int batc
             f.nw = w > f.nw ? w : f.nw;
             nbias = c > nbias ? c : nbias;
             f.l[k] = FinishLayer{gw.Z, m->dZ[l], m->woff[l], m->boff[l], m->dout[l], m->din[l], m->kpad[l], m->opad[l],
-                                 m->Wb[l], m->WTb[l]};
+                                 m->Wb[l], m->WTb[l], m->Wp + m->wpoff[l]};
         }
         k_wgrad<<<dim3(mt, nt, nl * gb.splits), GEMM_THREADS, gemm_smem_bytes(64), m->stream>>>(gb, 64);
         MCK(m, cudaGetLastError());
@@ -1059,7 +1327,7 @@ extern "C" int lbif_mlp_gradients(lbif_mlp m, const float* X, const float* T, co
         return mfail(m, LBIF_ERR_ARG, "lbif_mlp_gradients: bad arguments");
     int rc = pack_input(m, X, batch, on_device);
     if (rc) return rc;
-    if ((rc = forward(m, batch, true))) return rc;
+    if ((rc = forward(m, batch))) return rc;
     if ((rc = backward(m, T, mask, batch, on_device, loss))) return rc;
     if (grads) {
         MCK(m, cudaMemcpyAsync(grads, m->g, sizeof(float) * m->nparams,
@@ -1076,7 +1344,7 @@ extern "C" int lbif_mlp_train_step(lbif_mlp m, const float* X, const float* T, c
         return mfail(m, LBIF_ERR_ARG, "lbif_mlp_train_step: bad arguments");
     int rc = pack_input(m, X, batch, on_device);
     if (rc) return rc;
-    if ((rc = forward(m, batch, true))) return rc;
+    if ((rc = forward(m, batch))) return rc;
     // the update rides on the gradients' last kernel; a step whose products
     // failed leaves the parameters and the step count as they were
     const double t = (double)(m->adam_t + 1);
