@@ -189,6 +189,5 @@ cudaError_t launch_moments_out(const Params& P, const Fields& f, float* rho, flo
 // per-plane sums (dn, ux, (1+dn) ux, (1+dn) uy, (1+dn) uz), the rest is work space
 size_t profile_doubles(const Geom& g);
 cudaError_t launch_profiles(const Params& P, const Fields& f, double* prof, cudaStream_t s);
-bool force_vectorised(int sigma);
 
 }  // namespace lbif
