@@ -38,9 +38,9 @@ struct lbif_ctx {
     float* dG = nullptr;
     float4* Ft = nullptr;
     float4* F = nullptr;              // F / n0 per node (force kernel -> collision kernel)
-    int* tail_off = nullptr;
-    float4* tail_K = nullptr;
-    int tail_pairs = 0;
+    TailRow* tail_rows = nullptr;     // direct tail sum (no spectral path): its rows and coefficients
+    float4* tail_coef = nullptr;
+    int tail_nrows = 0;
     float2* tail_work = nullptr;      // spectral tail: fields, kernel transform, twiddles
     int tail_D = 0;                   // z reach of the tail kernel (planes)
     bool tail_fft = false;
@@ -164,7 +164,7 @@ static const CUtensorMap* ball_map(const lbif_ctx* h, int i)
 static cudaError_t run_tail(lbif_ctx* h, const float* dn)
 {
     if (h->tail_fft) return launch_tail_spectral(h->P, dn, h->tail_D, h->tail_work, h->Ft, h->stream);
-    return launch_tail(h->P, dn, h->tail_off, h->tail_K, h->tail_pairs, h->Ft, h->stream);
+    return launch_tail(h->P, dn, h->tail_rows, h->tail_nrows, h->tail_coef, h->Ft, h->stream);
 }
 
 // padded fields carry PAD_SLACK floats before their first element
@@ -199,7 +199,7 @@ static void free_ctx(lbif_ctx* h)
 {
     if (!h) return;
     if (h->graph) cudaGraphExecDestroy(h->graph);
-    void* bufs[] = {h->pop[0], h->pop[1], h->Ft, h->F, h->tail_off, h->tail_K, h->tail_work, h->status_d,
+    void* bufs[] = {h->pop[0], h->pop[1], h->Ft, h->F, h->tail_rows, h->tail_coef, h->tail_work, h->status_d,
                     h->prof_d, h->scratch, h->d_sl, h->d_zslit, h->d_done, h->clk_d};
     for (void* b : bufs)
         if (b) cudaFree(b);
@@ -280,6 +280,61 @@ static int build_shell(Params& P)
         }
     }
     return 0;
+}
+
+// phi'(r)/r of the Lennard-Jones tail
+static double tail_slope(int sigma, double eps, double r2)
+{
+    const double r = sqrt(r2), s6 = pow((double)sigma, 6.0), s12 = s6 * s6;
+    return 4.0 * eps * (-12.0 * s12 / pow(r, 13.0) + 6.0 * s6 / pow(r, 7.0)) / r;
+}
+
+// tail taps: one representative of each +-d pair with sigma <= |d| <= rcut sigma
+static void tail_pairs(int sigma, double rcut, double eps, std::vector<int>& dxs, std::vector<int>& dys,
+                       std::vector<int>& dzs, std::vector<float4>& K)
+{
+    const double rmax = rcut * sigma;
+    const int R = (int)ceil(rmax);
+    for (int dz = 0; dz <= R; ++dz)
+        for (int dy = (dz == 0 ? 0 : -R); dy <= R; ++dy)
+            for (int dx = ((dz == 0 && dy == 0) ? 1 : -R); dx <= R; ++dx) {
+                const double r2 = (double)dx * dx + (double)dy * dy + (double)dz * dz;
+                if (r2 < (double)sigma * sigma || r2 > rmax * rmax) continue;
+                const double k = tail_slope(sigma, eps, r2);
+                dxs.push_back(dx);
+                dys.push_back(dy);
+                dzs.push_back(dz);
+                K.push_back(make_float4((float)(k * dx), (float)(k * dy), (float)(k * dz), 0.f));
+            }
+}
+
+// the same displacements as rows for the direct sum (see TailRow)
+static void tail_direct_rows(const Geom& g, int sigma, double rcut, double eps, std::vector<TailRow>& rows,
+                             std::vector<float4>& coef)
+{
+    const double rmax = rcut * sigma;
+    const int R = (int)ceil(rmax);
+    for (int dz = 0; dz <= R; ++dz)
+        for (int dy = (dz == 0 ? 0 : -R); dy <= R; ++dy) {
+            std::vector<double> c(4 * (R / 4 + 1), 0.0);
+            int lo = -1, hi = -1;
+            for (int dx = 0; dx <= R; ++dx) {
+                const double r2 = (double)dx * dx + (double)dy * dy + (double)dz * dz;
+                if (r2 < (double)sigma * sigma || r2 > rmax * rmax) continue;
+                c[dx] = tail_slope(sigma, eps, r2);
+                if (dx == 0 || (dy == 0 && dz == 0)) c[dx] *= 0.5;
+                if (lo < 0) lo = dx / 4;
+                hi = dx / 4;
+            }
+            if (lo < 0) continue;
+            rows.push_back(TailRow{padded_offset(g, 0, dy, dz), (float)dy, (float)dz, lo, hi - lo + 1,
+                                   (int)coef.size()});
+            for (int j = 4 * lo; j < 4 * hi + 4; j += 4) {
+                coef.push_back(make_float4((float)c[j], (float)c[j + 1], (float)c[j + 2], (float)c[j + 3]));
+                coef.push_back(make_float4((float)(c[j] * j), (float)(c[j + 1] * (j + 1)), (float)(c[j + 2] * (j + 2)),
+                                           (float)(c[j + 3] * (j + 3))));
+            }
+        }
 }
 
 static int ball_count(int sigma)
@@ -429,30 +484,7 @@ static int create_impl(lbif_handle* out, int nx, int ny, int nz, int sigma, int 
         h->own_stream = true;
     }
 
-    // tail taps: one representative of each +-d pair with sigma <= |d| <= rcut sigma
-    std::vector<int> toff, tdx, tdy, tdz;
-    std::vector<float4> tK;
-    if (P.tail) {
-        double rmax = F.rcut * sigma;
-        int R = (int)ceil(rmax);
-        h->tail_D = R;
-        double s6 = pow((double)sigma, 6.0), s12 = s6 * s6;
-        for (int dz = 0; dz <= R; ++dz)
-            for (int dy = (dz == 0 ? 0 : -R); dy <= R; ++dy)
-                for (int dx = ((dz == 0 && dy == 0) ? 1 : -R); dx <= R; ++dx) {
-                    double r2 = (double)dx * dx + (double)dy * dy + (double)dz * dz;
-                    if (r2 < (double)sigma * sigma || r2 > rmax * rmax) continue;
-                    double r = sqrt(r2);
-                    double dphi = 4.0 * F.eps * (-12.0 * s12 / pow(r, 13.0) + 6.0 * s6 / pow(r, 7.0));
-                    toff.push_back(padded_offset(g, dx, dy, dz));
-                    tdx.push_back(dx);
-                    tdy.push_back(dy);
-                    tdz.push_back(dz);
-                    tK.push_back(make_float4((float)(dphi * dx / r), (float)(dphi * dy / r),
-                                             (float)(dphi * dz / r), 0.f));
-                }
-        h->tail_pairs = (int)toff.size();
-    }
+    if (P.tail) h->tail_D = (int)ceil(F.rcut * sigma);
 
     size_t pb = pop_bytes(P) * (size_t)Q * (size_t)g.Npad;
 #define ALLOC(ptr, bytes)                                                                   \
@@ -477,8 +509,6 @@ static int create_impl(lbif_handle* out, int nx, int ny, int nz, int sigma, int 
     ALLOC(h->d_done, sizeof(int) * h->sl.size());
     if (P.tail) {
         ALLOC(h->Ft, sizeof(float4) * (size_t)g.N);
-        ALLOC(h->tail_off, sizeof(int) * toff.size());
-        ALLOC(h->tail_K, sizeof(float4) * tK.size());
     }
 #undef ALLOC
     {
@@ -538,10 +568,11 @@ static int create_impl(lbif_handle* out, int nx, int ny, int nz, int sigma, int 
     }
     CKC(cudaMemsetAsync(h->status_d, 0, sizeof(int), h->stream));
     if (P.tail) {
-        CKC(cudaMemcpyAsync(h->tail_off, toff.data(), sizeof(int) * toff.size(),
-                            cudaMemcpyHostToDevice, h->stream));
         // spectral path when the lateral extents allow it; else the direct sum
         if (tail_spectral_ok(g)) {
+            std::vector<int> tdx, tdy, tdz;
+            std::vector<float4> tK;
+            tail_pairs(sigma, F.rcut, F.eps, tdx, tdy, tdz, tK);
             if (cudaMalloc((void**)&h->tail_work, tail_spectral_bytes(g, h->tail_D)) == cudaSuccess &&
                 tail_spectral_init(g, h->tail_D, tdx.data(), tdy.data(), tdz.data(), tK.data(), (int)tK.size(),
                                    h->zslit.data(), h->tail_work, h->stream) == cudaSuccess) {
@@ -552,8 +583,25 @@ static int create_impl(lbif_handle* out, int nx, int ny, int nz, int sigma, int 
                 h->tail_work = nullptr;
             }
         }
-        CKC(cudaMemcpyAsync(h->tail_K, tK.data(), sizeof(float4) * tK.size(),
-                            cudaMemcpyHostToDevice, h->stream));
+        if (!h->tail_fft) {
+            std::vector<TailRow> rows;
+            std::vector<float4> coef;
+            tail_direct_rows(g, sigma, F.rcut, F.eps, rows, coef);
+            h->tail_nrows = (int)rows.size();
+            // (never empty allocations)
+            cudaError_t e = cudaMalloc((void**)&h->tail_rows, sizeof(TailRow) * (rows.size() + 1));
+            if (e == cudaSuccess) e = cudaMalloc((void**)&h->tail_coef, sizeof(float4) * (coef.size() + 1));
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                free_ctx(h);
+                return alloc_failed(e);
+            }
+            CKC(cudaMemcpyAsync(h->tail_rows, rows.data(), sizeof(TailRow) * rows.size(), cudaMemcpyHostToDevice,
+                                h->stream));
+            CKC(cudaMemcpyAsync(h->tail_coef, coef.data(), sizeof(float4) * coef.size(), cudaMemcpyHostToDevice,
+                                h->stream));
+            CKC(cudaStreamSynchronize(h->stream));
+        }
     }
     CKC(launch_init_noise(P, h->dn[0], O.seed, O.noise, 0, h->stream));
     CKC(cudaStreamSynchronize(h->stream));

@@ -149,8 +149,18 @@ cudaError_t launch_ball(const Params& P, const float* dn, float* dG, int* status
                         int skip_done, cudaStream_t s, const CUtensorMap* tmap = nullptr);
 // box (x extent W, y extent H) of the ball kernel's plane tile for sigma
 void ball_box(int sigma, int* W, int* H);
-cudaError_t launch_tail(const Params& P, const float* dn, const int* off, const float4* K,
-                        int npairs, float4* Ft, cudaStream_t s);
+// one row (dy, dz) of the tail kernel's displacements (a half space of them):
+// padded offset of (0, dy, dz), the first chunk of four dx that holds a term
+// (|dx| = 4 first ..), the number of chunks, and where their coefficients
+// start: two float4 per chunk, phi'(|d|)/|d| and the same times dx, halved
+// where dx and -dx are the same displacement or the same pair
+struct TailRow {
+    int off;
+    float dy, dz;
+    int first, count, coef;
+};
+cudaError_t launch_tail(const Params& P, const float* dn, const TailRow* rows, int nrows, const float4* coef,
+                        float4* Ft, cudaStream_t s);
 // group: edge (nodes) of the x-y block the resident CTAs sweep together (<= 0: default)
 cudaError_t launch_force(const Params& P, const Fields& f, const float4* Ft, float4* F, int group,
                          cudaStream_t s);
