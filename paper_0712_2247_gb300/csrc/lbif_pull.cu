@@ -378,17 +378,18 @@ struct CsmStaged {
     int p[CSM_KS], n[CSM_KS];
 };
 
-template <int NT>
+template <int NT, int TX = CSM_TX>
 __device__ __forceinline__ CsmStaged csm_staged(const Geom& g, int x0, int y0)
 {
-    static_assert(NT * CSM_KS >= CSM_HN, "two staged nodes per thread at most");
+    constexpr int HX = TX + 2, HN = HX * (CSM_THREADS / TX + 2);
+    static_assert(NT * CSM_KS >= HN && HN <= CSM_HN, "two staged nodes per thread at most");
     CsmStaged st;
 #pragma unroll
     for (int k = 0; k < CSM_KS; ++k) {
         const int h = threadIdx.x + k * NT;
-        const int X = x0 - 1 + h % CSM_HX, Y = y0 - 1 + h / CSM_HX;
+        const int X = x0 - 1 + h % HX, Y = y0 - 1 + h / HX;
         st.p[k] = st.n[k] = -1;
-        if (h >= CSM_HN || X > g.nx || Y > g.ny) continue;
+        if (h >= HN || X > g.nx || Y > g.ny) continue;
         const int xw = X < 0 ? X + g.nx : (X >= g.nx ? X - g.nx : X);
         const int yw = Y < 0 ? Y + g.ny : (Y >= g.ny ? Y - g.ny : Y);
         st.p[k] = (Y + g.hw) * g.px + (X + g.hw);
@@ -628,7 +629,8 @@ __global__ void __launch_bounds__(CSM_THREADS, CSM_MINB)
 
 // ---- two planes at a time ------------------------------------------------
 // The default form: a thread owns the nodes (x, y, z) and (x, y, z + 1) and a
-// CTA marches its 32 x 4 tile up two planes per round. The pair's arithmetic
+// CTA marches its tile of 128 nodes (TX x 128 / TX, 32 x 4 on all but narrow
+// grids) up two planes per round. The pair's arithmetic
 // is paired FP32 (one instruction for both nodes), one shared-memory load
 // brings a staged quantity of both nodes, their wrapped x-y offsets are
 // computed once, and a round of two planes costs two barriers. Populations
@@ -717,12 +719,12 @@ struct PullPtrs {
     void* dst[Q];
 };
 
-template <typename T, bool IP>
+template <typename T, bool IP, int TX>
 __global__ void __launch_bounds__(CSM_THREADS, PAIR_MINB)
     k_pull_pair(Params P, PullPtrs pp, CsmIO io, const float4* __restrict__ F, int lz, int tiles_x, int tiles_y,
                 int* status)
 {
-    constexpr int NT = CSM_THREADS;
+    constexpr int NT = CSM_THREADS, TY = NT / TX, HX = TX + 2;
     constexpr bool RAW = F16_RAW<T>;
     extern __shared__ __align__(16) float2 psm[];
     float2* const AB = psm;
@@ -731,13 +733,13 @@ __global__ void __launch_bounds__(CSM_THREADS, PAIR_MINB)
     const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
     const int tiles = tiles_x * tiles_y;
     const int tile = blockIdx.x % tiles, seg = blockIdx.x / tiles;
-    const int x0 = (tile % tiles_x) * CSM_TX, y0 = (tile / tiles_x) * CSM_TY;
+    const int x0 = (tile % tiles_x) * TX, y0 = (tile / tiles_x) * TY;
     const int t = threadIdx.x;
-    const int x = x0 + t % CSM_TX, y = y0 + t / CSM_TX;
-    const int hc = (t / CSM_TX + 1) * CSM_HX + t % CSM_TX + 1;
+    const int x = x0 + t % TX, y = y0 + t / TX;
+    const int hc = (t / TX + 1) * HX + t % TX + 1;
     const bool in_xy = x < nx && y < ny;
     const int zb = seg * lz, ze = min(zb + lz, nz);
-    const CsmStaged st = csm_staged<NT>(g, x0, y0);
+    const CsmStaged st = csm_staged<NT, TX>(g, x0, y0);
     const int pplane = g.py * g.px;
     const bool shifted = P.shifted != 0;
 
@@ -751,7 +753,7 @@ __global__ void __launch_bounds__(CSM_THREADS, PAIR_MINB)
     auto stage_load = [&](int q, int k, PairStage& a) {
         a.d = a.ux = a.uy = a.uz = make_float2(0.f, 0.f);
         a.f0 = a.f1 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (k * NT >= CSM_HN || st.p[k] < 0) return;
+        if (st.p[k] < 0) return;
         const int p = (q + g.hw) * pplane + st.p[k];
         const int q0 = plane_of(q), q1 = plane_of(q + 1);
         if (q0 >= 0) {
@@ -772,7 +774,7 @@ __global__ void __launch_bounds__(CSM_THREADS, PAIR_MINB)
     // planes (q, q + 1) into pair slot ab; plane q completes own slot ow, plane
     // q + 1 begins the other
     auto stage_store = [&](int q, int k, const PairStage& a, int ab, int ow) {
-        if (k * NT >= CSM_HN || st.p[k] < 0) return;
+        if (st.p[k] < 0) return;
         const int h = t + k * NT;
         float2 om = make_float2(0.f, 0.f);
         if (shifted) {
@@ -894,7 +896,7 @@ __global__ void __launch_bounds__(CSM_THREADS, PAIR_MINB)
             const float2 dnr = make_float2(lo[AB_DN * CSM_HN].y, hi[AB_DN * CSM_HN].x);
             auto src = [&](auto ic) {
                 constexpr int i = decltype(ic)::value;
-                constexpr int o = -kCx(i) - kCy(i) * CSM_HX, cz = kCz(i);
+                constexpr int o = -kCx(i) - kCy(i) * HX, cz = kCz(i);
                 if constexpr (cz != 0)
                     return SideSrc{(cz > 0 ? lo : hi) + o};
                 else
@@ -939,7 +941,7 @@ __global__ void __launch_bounds__(CSM_THREADS, PAIR_MINB)
             const float* above = fh + j;
             auto src = [&](auto ic) {
                 constexpr int i = decltype(ic)::value;
-                constexpr int o = 2 * (-kCx(i) - kCy(i) * CSM_HX), cz = kCz(i);
+                constexpr int o = 2 * (-kCx(i) - kCy(i) * HX), cz = kCz(i);
                 return LoneSrc{fo + o, own + o, (cz > 0 ? below : (cz < 0 ? above : own)) + o};
             };
             const int s = j ? s1 : s0;
@@ -1109,71 +1111,88 @@ __global__ void __launch_bounds__(CSM_THREADS, 4)
     }
 }
 
-// a node's staged quantities in registers
-struct Terms {
-    float q[CSM_NF];
-    template <int K>
-    __device__ __forceinline__ float get() const
-    {
-        return q[K];
-    }
-    __device__ __forceinline__ float c0() const
-    {
-        return rest_term(q[SQ_CA], q[SQ_CA + 1], q[SQ_CA + 2], q[SQ_CP], q[SQ_CP + 1], q[SQ_CP + 2]);
-    }
-};
+// Thin grids (cross-sections of at most BLOCK_A nodes, such as the 4 x 4 slits
+// that generate training profiles): a marched tile would leave most threads
+// idle, so a CTA takes all nodes of tz whole planes, one per thread, with the
+// planes' staged quantities (and one plane below and above) in shared memory,
+// where the periodic neighbours in x and y are found by wrapping. The same code
+// forms and uses the quantities as in the marched forms (identical results).
+// 2048 slits of 4 x 4 x H: one node per thread without staging, each forming
+// its ~35 sources' quantities itself, 339 us; so 225 us.
+// (Writing the new moments through shared memory as whole padded planes, images
+// and all, instead of node by node: 217 us at 4 x 4, but 445 us against 372 at
+// 8 x 8; not kept.)
+constexpr int BLOCK_A = 64, BLOCK_NT = 256, BLOCK_NS = BLOCK_NT + 2 * BLOCK_A;
 
-// Narrow grids (below one 32 x 4 tile): the same pass with one thread per
-// node and no staging; every source's quantities are formed where they are
-// used, by the same code as the staged ones, so both kernels give identical
-// results.
 template <typename T, bool IP>
-__global__ void __launch_bounds__(128) k_pull_node(Params P, const T* pin, T* pout, CsmIO io,
-                                                   const float4* __restrict__ F, int* status)
+__global__ void __launch_bounds__(BLOCK_NT) k_pull_block(Params P, const T* pin, T* pout, CsmIO io,
+                                                         const float4* __restrict__ F, int tz, int* status)
 {
-    const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (idx >= P.g.N) return;
+    __shared__ float st[CSM_NF * BLOCK_NS];
+    constexpr bool RAW = F16_RAW<T>;
     const Geom& g = P.g;
-    int x, y, z;
-    decompose(g, idx, x, y, z);
-    const int s = slit_of(P, z);
-    if (s < 0 || frozen(P, s)) return;
-    const int zlo = P.sl[s].zlo, zhi = P.sl[s].zhi;
-    const float om = P.sl[s].inv_tau, om1s = (1.f - om) / store_scale<T>();
+    const int nx = g.nx, ny = g.ny, A = nx * ny, z0 = blockIdx.x * tz;
     const bool shifted = P.shifted != 0;
+    const int zl = threadIdx.x / A, xy = threadIdx.x - zl * A, y = xy / nx, x = xy - y * nx, z = z0 + zl;
+    const int s = zl < tz && z < g.nz ? slit_of(P, z) : -1;
+    const bool act = s >= 0 && !frozen(P, s);
+    const long long idx = (long long)z * A + xy;
     float v[Q];
     unsigned bb = 0;
     IpSlots q;
-    if constexpr (IP) q = ip_slots(P, P.sl[s], s, x, y, z);
-    csm_pull<0, Q, IP>(P, pin, idx, x, y, z, zlo, zhi, v, bb, q);
-    const int p = pidx(g, x, y, z);
-    auto terms_at = [&](int ps, long long nf) {
-        Terms t;
-        const float4 f = __ldg(F + nf);
-        src_terms(__ldg(io.dn + ps), __ldg(io.ux + ps), __ldg(io.uy + ps), __ldg(io.uz + ps), f.x, f.y, f.z, f.w, om,
-                  shifted, [&](int j, float val) { t.q[j] = val; });
-        return t;
-    };
-    const Terms own = terms_at(p, idx);
-    const float dnr = own.q[SQ_DN];
-    // the source quantities of direction i, formed where they are used
-    // (padded fields through their periodic images, the force at its
-    // wrapped node); walls never ask (they use own)
+    if (act) {
+        if constexpr (IP) q = ip_slots(P, P.sl[s], s, x, y, z);
+        csm_pull<0, Q, IP, T, RAW>(P, pin, idx, x, y, z, P.sl[s].zlo, P.sl[s].zhi, v, bb, q);
+    }
+    for (int k = threadIdx.x; k < (tz + 2) * A; k += blockDim.x) {
+        const int kz = k / A, kxy = k - kz * A, ky = kxy / nx, kx = kxy - ky * nx;
+        const int r = z0 - 1 + kz;  // plane; beyond a periodic end its image, beyond a wall nothing
+        const int w = g.zper ? (r < 0 ? r + g.nz : (r >= g.nz ? r - g.nz : r)) : r;
+        if (w < 0 || w >= g.nz || r > g.nz) continue;  // (the last CTA reaches past the grid)
+        const int ks = slit_of(P, w);
+        if (ks < 0 || frozen(P, ks)) continue;
+        const int p = pidx(g, kx, ky, r);
+        const float4 f = __ldg(F + ((long long)w * A + kxy));
+        src_terms(__ldg(io.dn + p), __ldg(io.ux + p), __ldg(io.uy + p), __ldg(io.uz + p), f.x, f.y, f.z, f.w,
+                  P.sl[ks].inv_tau, shifted, [&](int j, float val) { st[j * BLOCK_NS + k] = val; });
+    }
+    __syncthreads();
+    if (!act) return;
+    if constexpr (RAW) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) v[i] = late_cvt(v[i]);
+    }
+    const int xo[3] = {x, x > 0 ? x - 1 : nx - 1, x < nx - 1 ? x + 1 : 0};  // sources with c_x = 0, 1, -1
+    const int yo[3] = {y * nx, (y > 0 ? y - 1 : ny - 1) * nx, (y < ny - 1 ? y + 1 : 0) * nx};
+    using Src = Strided<BLOCK_NS>;
     auto src = [&](auto ic) {
         constexpr int i = decltype(ic)::value;
-        int sx = x - kCx(i), sy = y - kCy(i), sz = z - kCz(i);
-        sx = sx < 0 ? sx + g.nx : (sx >= g.nx ? sx - g.nx : sx);
-        sy = sy < 0 ? sy + g.ny : (sy >= g.ny ? sy - g.ny : sy);
-        if (g.zper) sz = sz < 0 ? sz + g.nz : (sz >= g.nz ? sz - g.nz : sz);
-        return terms_at(p - P.nbr[i], ((long long)sz * g.ny + sy) * g.nx + sx);
+        constexpr int cx = kCx(i), cy = kCy(i), cz = kCz(i);
+        return Src{st + (zl + 1 - cz) * A + yo[cy > 0 ? 1 : (cy < 0 ? 2 : 0)] + xo[cx > 0 ? 1 : (cx < 0 ? 2 : 0)]};
     };
-    float d79;
-    pull_gather_impl<true>(src, own, om1s, dnr, bb, v, d79);
-    float ux, uy, uz;
+    const Src own{st + (zl + 1) * A + xy};
+    const float dnr = own.get<SQ_DN>();
+    float d79, ux, uy, uz;
+    pull_gather(src, own, (1.f - P.sl[s].inv_tau) / store_scale<T>(), dnr, bb, v, d79);
     const float dn =
         pull_finish<T>([&](int i, float h) { stp(IP ? pop_at_ip(pout, P, i, q.slot(i)) : pop_at(pout, P, i, idx), h); },
                        v, d79, dnr, ux, uy, uz);
     put_fields(P, io, x, y, z, dn, ux, uy, uz, status);
+}
+
+template <typename T, bool IP>
+static cudaError_t pull_block(const Params& P, const void* pin, void* pout, const CsmIO& io, const float4* F,
+                              int* status, cudaStream_t s)
+{
+    const Geom& g = P.g;
+    const int A = g.nx * g.ny;
+    // planes per CTA: a full CTA, fewer on small grids so that the SMs share them
+    int tz = BLOCK_NT / A;
+    const int share = (g.nz + 2 * NUM_SMS - 1) / (2 * NUM_SMS);
+    if (tz > share) tz = share;
+    const int threads = (tz * A + 31) / 32 * 32;
+    k_pull_block<T, IP><<<(g.nz + tz - 1) / tz, threads, 0, s>>>(P, (const T*)pin, (T*)pout, io, F, tz, status);
+    return cudaGetLastError();
 }
 
 bool csm_ok(const Geom& g) { return g.nx >= CSM_TX && g.ny >= CSM_TY; }
@@ -1200,12 +1219,13 @@ static int pair_segment(long long tiles, int nz)
     return best;
 }
 
-template <typename T, bool IP>
+template <typename T, bool IP, int TX>
 static cudaError_t pull_pair(const Params& P, const void* pin, void* pout, const CsmIO& io, const float4* F,
                              int* status, int lz, cudaStream_t s)
 {
     const Geom& g = P.g;
-    const int tx = (g.nx + CSM_TX - 1) / CSM_TX, ty = (g.ny + CSM_TY - 1) / CSM_TY;
+    constexpr int TY = CSM_THREADS / TX;
+    const int tx = (g.nx + TX - 1) / TX, ty = (g.ny + TY - 1) / TY;
     if (lz <= 0) lz = pair_segment((long long)tx * ty, g.nz);
     lz += lz & 1;  // two planes per round
     const int segs = (g.nz + lz - 1) / lz;
@@ -1219,7 +1239,7 @@ static cudaError_t pull_pair(const Params& P, const void* pin, void* pout, const
     if (e != cudaSuccess) return e;
     const uint64_t bit = 1ull << (dev & 63);
     if (!(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(k_pull_pair<T, IP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k_pull_pair<T, IP, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         configured.fetch_or(bit);
     }
@@ -1231,8 +1251,42 @@ static cudaError_t pull_pair(const Params& P, const void* pin, void* pout, const
         pp.src[i] = static_cast<const T*>(pin) + P.dbase[i] + back;
         pp.dst[i] = static_cast<T*>(pout) + P.dbase[i];
     }
-    k_pull_pair<T, IP><<<(unsigned)blocks, CSM_THREADS, smem, s>>>(P, pp, io, F, lz, tx, ty, status);
+    k_pull_pair<T, IP, TX><<<(unsigned)blocks, CSM_THREADS, smem, s>>>(P, pp, io, F, lz, tx, ty, status);
     return cudaGetLastError();
+}
+
+// The tile's width: the one that covers the cross-section with the least work,
+// a tile of 16 or 8 columns counted 1.15 and 1.4 times one of 32 (its rows are
+// 64 or 32 bytes a warp load). With 32 / 16 / 8 columns: 203 x 117 x 75 112 / 121
+// / 154 us, a stack of 100 slits of 33 x 35 485 / 424 / 489 us, 7 x 300 x 100 50 /
+// 31 / 25 us, 100 slits of 48 x 24 (FP16 in place) 332 / 264 / 368 us.
+static int pair_width(const Geom& g)
+{
+    const int w[] = {32, 16, 8};
+    const double f[] = {1.0, 1.15, 1.4};
+    int best = 32;
+    double cost = 1e300;
+    for (int k = 0; k < 3; ++k) {
+        const int ty = CSM_THREADS / w[k];
+        const double c = f[k] * ((g.nx + w[k] - 1) / w[k]) * ((g.ny + ty - 1) / ty);
+        if (c < cost) {
+            cost = c;
+            best = w[k];
+        }
+    }
+    return best;
+}
+
+template <typename T, bool IP>
+static cudaError_t pull_any(const Params& P, const void* pin, void* pout, const CsmIO& io, const float4* F,
+                            int* status, int lz, cudaStream_t s)
+{
+    if ((long long)P.g.nx * P.g.ny <= BLOCK_A) return pull_block<T, IP>(P, pin, pout, io, F, status, s);
+    switch (pair_width(P.g)) {
+    case 32: return pull_pair<T, IP, 32>(P, pin, pout, io, F, status, lz, s);
+    case 16: return pull_pair<T, IP, 16>(P, pin, pout, io, F, status, lz, s);
+    default: return pull_pair<T, IP, 8>(P, pin, pout, io, F, status, lz, s);
+    }
 }
 
 template <typename T, bool IP>
@@ -1295,20 +1349,12 @@ cudaError_t launch_csm(const Params& P, const void* pin, void* pout, const CsmIO
         return h16 ? csm_tma<__half>(P, pmap, pin, pout, io, F, status, lz, s)
                    : csm_tma<float>(P, pmap, pin, pout, io, F, status, lz, s);
     }
-    if (!csm_ok(g)) {
-        const unsigned nb = nblocks(g.N, 128);
-        if (h16 && ip) k_pull_node<__half, true><<<nb, 128, 0, s>>>(P, (const __half*)pin, (__half*)pout, io, F, status);
-        if (h16 && !ip) k_pull_node<__half, false><<<nb, 128, 0, s>>>(P, (const __half*)pin, (__half*)pout, io, F, status);
-        if (!h16 && ip) k_pull_node<float, true><<<nb, 128, 0, s>>>(P, (const float*)pin, (float*)pout, io, F, status);
-        if (!h16 && !ip) k_pull_node<float, false><<<nb, 128, 0, s>>>(P, (const float*)pin, (float*)pout, io, F, status);
-        return cudaGetLastError();
-    }
-    if (prefetch != 1) {
+    if (prefetch != 1 || !csm_ok(g)) {
         if (h16)
-            return ip ? pull_pair<__half, true>(P, pin, pout, io, F, status, lz, s)
-                      : pull_pair<__half, false>(P, pin, pout, io, F, status, lz, s);
-        return ip ? pull_pair<float, true>(P, pin, pout, io, F, status, lz, s)
-                  : pull_pair<float, false>(P, pin, pout, io, F, status, lz, s);
+            return ip ? pull_any<__half, true>(P, pin, pout, io, F, status, lz, s)
+                      : pull_any<__half, false>(P, pin, pout, io, F, status, lz, s);
+        return ip ? pull_any<float, true>(P, pin, pout, io, F, status, lz, s)
+                  : pull_any<float, false>(P, pin, pout, io, F, status, lz, s);
     }
     if (lz <= 0) lz = CSM_LZ;
     if (h16)
