@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_wgrad(const __grid_constant
 // per element against 512 FLOP on the tensor core, so two CTAs share an SM and
 // one's epilogue covers the other's products. Four launches that passed the
 // activations through L2 took 234 us for 65,536 rows at 4 -> 3 x 256 -> 160; this
-// takes 138 us, 115 of them in the kernel (43 us of issue; an SM holds three or
+// takes 134 us, 115 of them in the kernel (43 us of issue; an SM holds three or
 // four of the 512 tiles). Loading the next chunk of accumulators and biases
 // early changed nothing.
 // ---------------------------------------------------------------------------
@@ -437,6 +437,7 @@ struct Fused {
     int batch, nin, hidden, nout, L;
     int tiles, achunk;  // row tiles; bytes of the activation buffer
     int* err;
+    double* herr;     // what the host reads (mapped host memory)
 };
 
 __device__ __forceinline__ bool bounded_wait(uint64_t* mbar, uint32_t parity)
@@ -623,6 +624,7 @@ __global__ void __launch_bounds__(256, 2) k_mlp_forward(const __grid_constant__ 
     }
     if (!ok && tid == 0) {
         atomicExch(f.err, 1);
+        *f.herr = 1.0;
         // copies in flight land before the CTA leaves
         for (long long q = nmma; q < nload; ++q)
             bounded_wait(full + (int)(q % FUSE_RING), (uint32_t)(q / FUSE_RING) & 1u);
@@ -819,7 +821,7 @@ __global__ void __launch_bounds__(256) k_finish(const __grid_constant__ Finish f
         const double ms = t < 32 ? mask_sum(f.mpart) : 1.0;
         if (t == 0) {
             f.result[0] = s / ms;
-            f.result[1] = (double)*f.err;
+            if (*f.err) f.result[1] = 1.0;
         }
         return;
     }
@@ -886,7 +888,10 @@ struct lbif_mlp_ctx {
     float *Td = nullptr, *Md = nullptr, *Yd = nullptr;
     double* partial = nullptr;
     double* mpart = nullptr;
-    double* result = nullptr;    // {loss, err} of a training call
+    // {loss, err} as the host reads them after a synchronisation: mapped host
+    // memory that the kernels write, so that no call ends with a copy (a 4-byte
+    // read-back took 10 us of each)
+    double *host = nullptr, *result = nullptr;  // host and device address
     int* err = nullptr;
     long long adam_t = 0;
     std::string msg;
@@ -924,7 +929,7 @@ static int mfail(lbif_mlp_ctx* m, int code, const std::string& s)
 static void mlp_free(lbif_mlp_ctx* m)
 {
     if (!m) return;
-    std::vector<void*> bufs = {m->Wp, m->p, m->g, m->m, m->v, m->dY, m->dWpart, m->Xd, m->Td, m->Md, m->Yd, m->partial, m->mpart, m->result, m->err};
+    std::vector<void*> bufs = {m->Wp, m->p, m->g, m->m, m->v, m->dY, m->dWpart, m->Xd, m->Td, m->Md, m->Yd, m->partial, m->mpart, m->err};
     for (auto* b : m->Wb) bufs.push_back(b);
     for (auto* b : m->WTb) bufs.push_back(b);
     for (auto* b : m->Z) bufs.push_back(b);
@@ -935,6 +940,7 @@ static void mlp_free(lbif_mlp_ctx* m)
     for (auto* b : m->dZT) bufs.push_back(b);
     for (void* b : bufs)
         if (b) cudaFree(b);
+    if (m->host) cudaFreeHost(m->host);
     delete m;
 }
 
@@ -997,7 +1003,7 @@ extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32
               dalloc(&m->Xd, (size_t)max_batch * nin) && dalloc(&m->Td, (size_t)max_batch * nout) &&
               dalloc(&m->Md, (size_t)max_batch * nout) && dalloc(&m->Yd, (size_t)bp * nout) &&
               dalloc(&m->partial, (size_t)(bp * nout + 255) / 256 + 1) && dalloc(&m->mpart, MSUM_BLOCKS) &&
-              dalloc(&m->result, 2) && dalloc(&m->err, 1) && dalloc(&m->Wp, npack);
+              dalloc(&m->err, 1) && dalloc(&m->Wp, npack);
     for (int l = 0; ok && l < m->L; ++l) {
         bf16 *wb, *wtb, *h, *ht, *dzb, *dzt;
         float *z, *dz;
@@ -1014,7 +1020,11 @@ extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32
         m->dZb.push_back(ok ? dzb : nullptr);
         m->dZT.push_back(ok ? dzt : nullptr);
     }
+    ok = ok && cudaHostAlloc((void**)&m->host, 2 * sizeof(double), cudaHostAllocMapped) == cudaSuccess &&
+         cudaHostGetDevicePointer((void**)&m->result, m->host, 0) == cudaSuccess;
+    if (ok) m->host[0] = m->host[1] = 0.0;
     if (!ok) {
+        cudaGetLastError();
         mlp_free(m);
         return mfail(nullptr, LBIF_ERR_NOMEM, "lbif_mlp_create: device allocation failed");
     }
@@ -1151,6 +1161,7 @@ static int infer(lbif_mlp_ctx* m, const float* X, int batch, float* Y)
     const int nmax = m->opad[m->L - 1] > m->hidden ? m->opad[m->L - 1] : m->hidden;
     f.achunk = 256 * kmax;
     f.err = m->err;
+    f.herr = m->result + 1;
     // two CTAs per SM: shared memory keeps a third one (and its TMEM) out
     int smem = fused_smem(kmax, nmax);
     if (smem < 80 * 1024) smem = 80 * 1024;
@@ -1176,10 +1187,8 @@ static int pack_input(lbif_mlp_ctx* m, const float* X, int batch, int on_device)
 
 static int check_err(lbif_mlp_ctx* m)
 {
-    int e = 0;
-    MCK(m, cudaMemcpyAsync(&e, m->err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
     MCK(m, cudaStreamSynchronize(m->stream));
-    if (e) return mfail(m, LBIF_ERR_TIMEOUT, "tensor-core product did not complete within its wait limit");
+    if (*(volatile double*)(m->host + 1) != 0.0) return mfail(m, LBIF_ERR_TIMEOUT, "tensor-core product did not complete within its wait limit");
     return LBIF_OK;
 }
 
@@ -1311,12 +1320,9 @@ static int backward(lbif_mlp_ctx* m, const float* T, const float* mask, int batc
         k_finish<<<fgrid[k], 256, 0, m->stream>>>(fin[k]);
         MCK(m, cudaGetLastError());
     }
-    double r[2] = {0.0, 0.0};
-    MCK(m, cudaMemcpyAsync(r, m->result, 2 * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
-    MCK(m, cudaStreamSynchronize(m->stream));
-    if (r[1] != 0.0)
-        return mfail(m, LBIF_ERR_TIMEOUT, "tensor-core product did not complete within its wait limit");
-    if (loss) *loss = r[0];
+    const int rc = check_err(m);
+    if (rc) return rc;
+    if (loss) *loss = *(volatile double*)m->host;
     return LBIF_OK;
 }
 
