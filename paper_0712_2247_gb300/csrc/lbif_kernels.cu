@@ -201,16 +201,13 @@ __device__ __forceinline__ float g2_deviation(const Params& P, float e0, float d
     return (dN * D0 - N0 * dD) / (D1 * D0);
 }
 
-// tile of the z-marching ball kernel: 32 x 16 nodes, 256 threads, each
-// thread a column of BALL_YT = 2 nodes in y (measured at sigma = 12 on a
-// 512 x 512 x 192 slit: 1 node per thread 0.86 ms, 2 nodes 0.72 ms, 4 nodes
-// 0.90 ms, each with its best CTA count; with tensor-memory-accelerator
-// staging, CTAs of 4 / 8 / 16 warps 0.567 / 0.552 / 0.573 ms)
-#ifndef BALL_WARPS
-#define BALL_WARPS 8
-#endif
-constexpr int BALL_TX = 32, BALL_YT = 2, BALL_TY = BALL_WARPS * BALL_YT, BALL_THREADS = 32 * BALL_WARPS;
-
+// tile of the z-marching ball kernel: 32 x 16 nodes, 256 threads, each thread
+// the columns of two x-adjacent nodes, whose disc sums one paired addition
+// serves (sigma 12 on 512 x 512 x 192, 1216 CTAs: two y-adjacent nodes with scalar
+// additions 0.554 ms, two x-adjacent ones paired 0.535 ms; 256 slits of 32 x 32,
+// sigma 4, 0.115 -> 0.105 ms; CTAs of 4 / 8 / 16 warps ran 0.567 / 0.552 / 0.573 ms
+// in the former form)
+constexpr int BALL_TX = 32, BALL_TY = 16, BALL_THREADS = BALL_TX / 2 * BALL_TY;
 
 // x halo of the staged plane tile: R rounded up to 4, so that tile rows and
 // their global sources are float4-aligned
@@ -241,54 +238,46 @@ __global__ void k_wait_selftest(long long polls, int* status)
     if (!__syncthreads_and(ok) && threadIdx.x == 0) atomicOr(status, 4);
 }
 
-// does tile row r (relative to a thread's first node row minus R) enter a
-// disc sum D_k of any of the thread's BALL_YT nodes with row half-width w?
+// does the row at dy = r - R enter a disc sum D_k with row half-width w?
 __host__ __device__ constexpr bool ball_row_used(int R, int r, int w)
 {
-    for (int j = 0; j < BALL_YT; ++j) {
-        const int dy = r - R - j;
-        if (dy < -R || dy > R) continue;
-        for (int k = 0; k <= R; ++k) {
-            const int rem = R * R - k * k - dy * dy;
-            if (rem >= 0 && cisqrt(rem) == w) return true;
-        }
+    for (int k = 0; k <= R; ++k) {
+        const int rem = R * R - k * k - (r - R) * (r - R);
+        if (rem >= 0 && cisqrt(rem) == w) return true;
     }
     return false;
 }
 
-// Compile-time expansion of the disc sums of one thread: for every tile row r
-// (in increasing order) and half-width w that some D[k][i] uses, one shared
-// memory read, added into exactly those D[k][i].
-template <int R, int r, int w, int M>
-__device__ __forceinline__ void ball_add_one(float v, float (&D)[R + 1][BALL_YT])
+// Compile-time expansion of the disc sums of one thread: for every row r (in
+// increasing order) and half-width w that some D[k] uses, one shared-memory
+// read of the two columns' row sums, added into exactly those D[k].
+template <int R, int r, int w, int k>
+__device__ __forceinline__ void ball_add_one(float2 v, float2 (&D)[R + 1])
 {
-    constexpr int i = M / (R + 1), k = M % (R + 1);
-    constexpr int dy = r - R - i;
-    constexpr int rem = R * R - k * k - dy * dy;
-    if constexpr (dy >= -R && dy <= R && rem >= 0 && cisqrt(rem) == w) D[k][i] += v;
+    constexpr int dy = r - R, rem = R * R - k * k - dy * dy;
+    if constexpr (rem >= 0 && cisqrt(rem) == w) D[k] = __fadd2_rn(D[k], v);
 }
 
-template <int R, int r, int w, int... M>
-__device__ __forceinline__ void ball_add_row(float v, float (&D)[R + 1][BALL_YT],
-                                             std::integer_sequence<int, M...>)
+template <int R, int r, int w, int... K>
+__device__ __forceinline__ void ball_add_row(float2 v, float2 (&D)[R + 1], std::integer_sequence<int, K...>)
 {
-    (ball_add_one<R, r, w, M>(v, D), ...);
+    (ball_add_one<R, r, w, K>(v, D), ...);
 }
 
 template <int R, int N>
-__device__ __forceinline__ void ball_disc_row(const float* __restrict__ RS, int off, float (&D)[R + 1][BALL_YT])
+__device__ __forceinline__ void ball_disc_row(const float* __restrict__ RS, int off, float2 (&D)[R + 1])
 {
     constexpr int r = N / (R + 1), w = N % (R + 1);
     constexpr int H = BALL_TY + 2 * R;
     if constexpr (ball_row_used(R, r, w)) {
-        const float v = RS[(w * H + r) * BALL_TX + off];
-        ball_add_row<R, r, w>(v, D, std::make_integer_sequence<int, BALL_YT * (R + 1)>{});
+        const float2 v = *reinterpret_cast<const float2*>(RS + (w * H + r) * BALL_TX + off);
+        ball_add_row<R, r, w>(v, D, std::make_integer_sequence<int, R + 1>{});
     }
 }
 
 // the comma fold runs the rows in increasing order
 template <int R, int... N>
-__device__ __forceinline__ void ball_disc_rows(const float* __restrict__ RS, int off, float (&D)[R + 1][BALL_YT],
+__device__ __forceinline__ void ball_disc_rows(const float* __restrict__ RS, int off, float2 (&D)[R + 1],
                                                std::integer_sequence<int, N...>)
 {
     (ball_disc_row<R, N>(RS, off, D), ...);
@@ -329,61 +318,53 @@ __device__ __forceinline__ void ball_rowsums(const float* __restrict__ T, float*
     }
 }
 
-// Disc sums of input plane zi for the thread's BALL_YT nodes, added into the
-// register ring acc of the 2R+1 output planes they touch; the completed plane
-// zi - R is written (g2 deviation, with its periodic images), the ring shifts.
+// Disc sums of input plane zi for the thread's two nodes (x, x + 1; y), added
+// into the register ring acc of the 2R+1 output planes they touch; the completed
+// plane zi - R is written (g2 deviation, with its periodic images), the ring
+// shifts.
 template <int R>
-__device__ __forceinline__ void ball_disc_out(const Params& P, const float* __restrict__ RS,
-                                              float (&acc)[2 * R + 1][BALL_YT], int zi, int z0, int x,
-                                              int y0, int ty0, int tx, float* __restrict__ dG, int* status,
-                                              int skip_done)
+__device__ __forceinline__ void ball_disc_out(const Params& P, const float* __restrict__ RS, float2 (&acc)[2 * R + 1],
+                                              int zi, int z0, int x, int y, int off, float* __restrict__ dG,
+                                              int* status, int skip_done)
 {
-    constexpr int YT = BALL_YT, TX = BALL_TX;
     const Geom& g = P.g;
-    // D[k][i] = sum over dy = -R..R (in that order) of the row sum of
-    // half-width cisqrt(R^2 - k^2 - dy^2) at row ty0 + i + dy
-    float D[R + 1][YT];
+    // D[k] = sum over dy = -R..R (in that order) of the row sum of half-width
+    // cisqrt(R^2 - k^2 - dy^2) at row y + dy
+    float2 D[R + 1];
 #pragma unroll
-    for (int k = 0; k <= R; ++k)
+    for (int k = 0; k <= R; ++k) D[k] = make_float2(0.f, 0.f);
+    ball_disc_rows<R>(RS, off, D, std::make_integer_sequence<int, (2 * R + 1) * (R + 1)>{});
 #pragma unroll
-        for (int i = 0; i < YT; ++i) D[k][i] = 0.f;
-    ball_disc_rows<R>(RS, ty0 * TX + tx, D, std::make_integer_sequence<int, (YT + 2 * R) * (R + 1)>{});
-#pragma unroll
-    for (int k = 0; k <= R; ++k)
-#pragma unroll
-        for (int i = 0; i < YT; ++i) {
-            acc[R - k][i] += D[k][i];
-            if (k) acc[R + k][i] += D[k][i];
-        }
+    for (int k = 0; k <= R; ++k) {
+        acc[R - k] = __fadd2_rn(acc[R - k], D[k]);
+        if (k) acc[R + k] = __fadd2_rn(acc[R + k], D[k]);
+    }
     const int zo = zi - R;
     const int so = zo >= z0 ? slit_of(P, zo) : -1;
-    if (so >= 0 && x < g.nx && !(skip_done && frozen(P, so))) {
+    if (so >= 0 && x < g.nx && y < g.ny && !(skip_done && frozen(P, so))) {
         const float e0 = P.sl[so].eta0;
-#pragma unroll
-        for (int i = 0; i < YT; ++i) {
-            const int y = y0 + ty0 + i;
-            if (y >= g.ny) break;
-            bool bad;
-            float v = g2_deviation(P, e0, acc[0][i] * P.ball_inv, bad);
-            if (bad) atomicOr(status, 2);
-            if (no_images(g, x, y, zo))
-                dG[pidx(g, x, y, zo)] = v;
-            else
-                for_images(g, x, y, zo, [&](int q) { dG[q] = v; });
+        bool bad0, bad1;
+        const float2 v = make_float2(g2_deviation(P, e0, acc[0].x * P.ball_inv, bad0),
+                                     g2_deviation(P, e0, acc[0].y * P.ball_inv, bad1));
+        const bool two = x + 1 < g.nx;
+        if (bad0 || (two && bad1)) atomicOr(status, 2);
+        if (two && no_images(g, x, y, zo) && no_images(g, x + 1, y, zo)) {
+            // x, hw and px even: 8-byte aligned
+            *reinterpret_cast<float2*>(dG + pidx(g, x, y, zo)) = v;
+        } else {
+            for_images(g, x, y, zo, [&](int q) { dG[q] = v.x; });
+            if (two) for_images(g, x + 1, y, zo, [&](int q) { dG[q] = v.y; });
         }
     }
 #pragma unroll
-    for (int j = 0; j < 2 * R; ++j)
-#pragma unroll
-        for (int i = 0; i < YT; ++i) acc[j][i] = acc[j + 1][i];
-#pragma unroll
-    for (int i = 0; i < YT; ++i) acc[2 * R][i] = 0.f;
+    for (int j = 0; j < 2 * R; ++j) acc[j] = acc[j + 1];
+    acc[2 * R] = make_float2(0.f, 0.f);
 }
 
 // One CTA = a 32 x 16 column of nodes marching up a z chunk. Per input plane:
 // stage the plane (+R halo) in shared memory, build x-row sums of every
 // half-width 0..R, form the disc sums D_k (disc of radius^2 R^2 - k^2; a
-// thread reads each row sum it needs once for its two nodes in y) and add
+// thread reads each row sum it needs once for its two nodes) and add
 // them into a register ring of the 2R+1 output planes they touch, emit the
 // completed plane.
 template <int R>
@@ -401,14 +382,11 @@ __global__ void __launch_bounds__(BALL_THREADS) k_ball(Params P, const float* __
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int z0 = blockIdx.z * zchunk;
     const int z1 = min(z0 + zchunk, g.nz);
-    constexpr int YT = BALL_YT;
-    const int tx = threadIdx.x % TX, ty0 = (threadIdx.x / TX) * YT;
-    const int x = x0 + tx;
-    float acc[2 * R + 1][YT];
+    const int tx = 2 * (threadIdx.x % (TX / 2)), ty = threadIdx.x / (TX / 2);
+    const int x = x0 + tx, y = y0 + ty, off = ty * TX + tx;
+    float2 acc[2 * R + 1];
 #pragma unroll
-    for (int j = 0; j <= 2 * R; ++j)
-#pragma unroll
-        for (int i = 0; i < YT; ++i) acc[j][i] = 0.f;
+    for (int j = 0; j <= 2 * R; ++j) acc[j] = make_float2(0.f, 0.f);
 
     for (int zi = z0 - R; zi < z1 + R; ++zi) {
         const float* plane = dn + (long long)(zi + g.hw) * g.py * g.px;
@@ -425,7 +403,7 @@ __global__ void __launch_bounds__(BALL_THREADS) k_ball(Params P, const float* __
         __syncthreads();
         ball_rowsums<R>(T, RS);
         __syncthreads();
-        ball_disc_out<R>(P, RS, acc, zi, z0, x, y0, ty0, tx, dG, status, skip_done);
+        ball_disc_out<R>(P, RS, acc, zi, z0, x, y, off, dG, status, skip_done);
         __syncthreads();
     }
 }
@@ -451,9 +429,8 @@ __global__ void __launch_bounds__(BALL_THREADS) k_ball_tma(Params P, const __gri
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int z0 = blockIdx.z * zchunk;
     const int z1 = min(z0 + zchunk, g.nz);
-    constexpr int YT = BALL_YT;
-    const int tx = threadIdx.x % TX, ty0 = (threadIdx.x / TX) * YT;
-    const int x = x0 + tx;
+    const int tx = 2 * (threadIdx.x % (TX / 2)), ty = threadIdx.x / (TX / 2);
+    const int x = x0 + tx, y = y0 + ty, off = ty * TX + tx;
     const int np = (z1 + R) - (z0 - R);  // input planes of this chunk
     // box origin in padded coordinates; x0 - C4 + hw is a multiple of 4 (16 bytes)
     const int bx = x0 - C4 + g.hw, by = y0 - R + g.hw;
@@ -480,11 +457,9 @@ __global__ void __launch_bounds__(BALL_THREADS) k_ball_tma(Params P, const __gri
         issue(0);
         if (np > 1) issue(1);
     }
-    float acc[2 * R + 1][YT];
+    float2 acc[2 * R + 1];
 #pragma unroll
-    for (int j = 0; j <= 2 * R; ++j)
-#pragma unroll
-        for (int i = 0; i < YT; ++i) acc[j][i] = 0.f;
+    for (int j = 0; j <= 2 * R; ++j) acc[j] = make_float2(0.f, 0.f);
     uint32_t pbits = 0u;  // bit b: phase parity expected next on buffer b
     for (int q = 0; q < np; ++q) {
         const int b = q & 1;
@@ -508,7 +483,7 @@ __global__ void __launch_bounds__(BALL_THREADS) k_ball_tma(Params P, const __gri
         ball_rowsums<R>(reinterpret_cast<const float*>(bsm + b * TB), RS);
         __syncthreads();  // buffer b is read: refill it two planes ahead
         if (threadIdx.x == 0 && q + 2 < np) issue(q + 2);
-        ball_disc_out<R>(P, RS, acc, z0 - R + q, z0, x, y0, ty0, tx, dG, status, skip_done);
+        ball_disc_out<R>(P, RS, acc, z0 - R + q, z0, x, y, off, dG, status, skip_done);
         __syncthreads();
     }
 }
@@ -894,9 +869,20 @@ static cudaError_t ball_r(const Params& P, const float* dn, float* dG, int* stat
         flags.fetch_or(bit);
     }
     int gx = (g.nx + BALL_TX - 1) / BALL_TX, gy = (g.ny + BALL_TY - 1) / BALL_TY;
-    if (want <= 0) want = 608;  // ~4 CTAs per SM on 152 SMs
+    // CTAs to aim for: about eight per SM (512 x 512 x 192, sigma 12: 608 / 1216 /
+    // 2432 / 4864 CTAs 0.606 / 0.554 / 0.564 / 0.625 ms in the former form; 256 x
+    // 256 x 128, sigma 8: 100 / 95 / 103 / 103 us). A chunk of z planes reads 2 R
+    // more, so chunks hold at least 2 R planes, unless that leaves fewer than three
+    // CTAs per SM (then R: 64 x 64 x 128, sigma 8, 24 -> 20 us; 256 x 256 x 64,
+    // sigma 10, with enough of them would lose 73 -> 80) or that fewer than one
+    // (then R / 2: 32 x 32 x 64, sigma 8, 23 / 16 / 14 us).
+    if (want <= 0) want = 8 * NUM_SMS;
     int nchunk = (want + gx * gy - 1) / (gx * gy);
-    int maxchunk = g.nz / (2 * R) > 1 ? g.nz / (2 * R) : 1;
+    const long long tiles = (long long)gx * gy;
+    int least = 2 * R;
+    if (tiles * (g.nz / least) < 3 * NUM_SMS) least = R;
+    if (tiles * (g.nz / least) < NUM_SMS) least = (R + 1) / 2;
+    const int maxchunk = g.nz / least > 1 ? g.nz / least : 1;
     if (nchunk > maxchunk) nchunk = maxchunk;
     if (nchunk < 1) nchunk = 1;
     int zchunk = (g.nz + nchunk - 1) / nchunk;
