@@ -1,5 +1,7 @@
 // Hard-sphere shell force (Eq. LBHS): the per-node kernel for any even sigma and
 // the vectorised one, with their launcher.
+#include <utility>
+
 #include "lbif_device.cuh"
 
 namespace lbif {
@@ -619,6 +621,153 @@ __global__ void __launch_bounds__(FORCE_NT, FORCE_MINB) k_force4(Params P, TileM
         const float c2 = C2 && P.hs ? 0.5f * pre * cc[j] : 0.f;
         F[idx0 + j] = make_float4(fx, fy, fz, c2);
     }
+}
+
+// ---------------------------------------------------------------------------
+// Local pressure p = kT n + (kT sigma^3/6) 4 pi n0^2 (1 + dn) sum_q W_q (G0 + A_q),
+// four consecutive x nodes per thread with the windows of the force kernel (n and
+// g2 only: half of its loads). 256 x 192 x 96, sigma 8: one node per thread with
+// scalar loads 159 us, so 74 us.
+// ---------------------------------------------------------------------------
+// acc += w0 c0 + w1 c1
+__device__ __forceinline__ void lerp4(float w0, float w1, const v4 c0, const v4 c1, v4 acc)
+{
+#pragma unroll
+    for (int j = 0; j < 4; j += 2) put2(acc, j, fma2(bc2(w1), p2(c1, j), fma2(bc2(w0), p2(c0, j), p2(acc, j))));
+}
+// s += W (G0 dq + gq (1 + dq))
+__device__ __forceinline__ void add_A(float W, const v4 dq, const v4 gq, float G0, v4 s)
+{
+#pragma unroll
+    for (int j = 0; j < 4; j += 2) put2(s, j, fma2(bc2(W), shell_A2(p2(dq, j), p2(gq, j), G0), p2(s, j)));
+}
+
+template <int SIG, bool LN>
+__global__ void __launch_bounds__(FORCE_NT) k_pressure4(Params P, TileMap tm, Fields fl, float* __restrict__ pr)
+{
+    const Geom& g = P.g;
+    int x, y, z;
+    bool live = true;
+    Lanes ln{false, false};
+    if (!LN) {
+        if (!flat_node(g, tm, 4, x, y, z)) return;
+    } else {
+        int tx, ty;
+        if (!tile_origin(g, tm, tx, ty, z)) return;
+        const int x0 = tx * 128, lane = threadIdx.x % 32;
+        x = x0 + 4 * lane;
+        y = ty * tm.ty + threadIdx.x / 32;
+        if (x0 >= g.nx || y >= g.ny) return;  // whole warp
+        live = x < g.nx;
+        if (!live) x = x0;
+        ln.hi = lane == 31 || x + 4 >= g.nx;
+        ln.lo = lane == 0;
+    }
+    const long long idx0 = ((long long)z * g.ny + y) * g.nx + x;
+    const int sl = slit_of(P, z);
+    if (sl < 0) {  // whole warp in the tiled mapping (one z plane)
+        if (live)
+            for (int j = 0; j < 4 && x + j < g.nx; ++j) pr[idx0 + j] = 0.f;
+        return;
+    }
+    const SlitParam S = P.sl[sl];
+    const int pb = pidx(g, x, y, z), sy = g.px, sz = g.px * g.py;
+    v4 d0, s;
+    set4(d0, ld4(fl.dn + pb));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s[j] = 0.f;
+    if (P.hs) {
+        constexpr int LO = cisqrt(SIG * SIG / 2), LOM = cisqrt((SIG / 2) * (SIG / 2) / 2);
+        v4 d, q;
+        win<SIG>(fl.dn, pb, d);
+        win<SIG / 2>(fl.dG, pb, q);
+        add_A(1.f / 30.f, d, q, S.G0, s);
+        win<-SIG>(fl.dn, pb, d);
+        win<-SIG / 2>(fl.dG, pb, q);
+        add_A(1.f / 30.f, d, q, S.G0, s);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int st = ((k & 1) ? -1 : 1) * ((k & 2) ? sz : sy);
+            set4(d, ld4(fl.dn + pb + SIG * st));
+            set4(q, ld4(fl.dG + pb + SIG / 2 * st));
+            add_A(1.f / 30.f, d, q, S.G0, s);
+        }
+        // planes (x, y) and (x, z): corners along x from the windows
+        auto member = [&](auto plc, auto sac, int sb) {
+            constexpr int PL = decltype(plc)::value, SA = decltype(sac)::value;
+            const int st = sb * (PL == 0 ? sy : sz);
+            v4 dq, gq, c0, c1;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) dq[j] = gq[j] = 0.f;
+#pragma unroll
+            for (int kb = 0; kb < 2; ++kb) {
+                corners_x<LO, SA, LN>(fl.dn, pb + (LO + kb) * st, c0, c1, ln);
+                lerp4(P.sh.nb_w[PL][2 * kb], P.sh.nb_w[PL][2 * kb + 1], c0, c1, dq);
+                corners_x<LOM, SA, LN>(fl.dG, pb + (LOM + kb) * st, c0, c1, ln);
+                lerp4(P.sh.md_w[PL][2 * kb], P.sh.md_w[PL][2 * kb + 1], c0, c1, gq);
+            }
+            add_A(1.f / 15.f, dq, gq, S.G0, s);
+        };
+        using std::integral_constant;
+#pragma unroll
+        for (int sb = -1; sb <= 1; sb += 2) {
+            member(integral_constant<int, 0>{}, integral_constant<int, 1>{}, sb);
+            member(integral_constant<int, 0>{}, integral_constant<int, -1>{}, sb);
+            member(integral_constant<int, 1>{}, integral_constant<int, 1>{}, sb);
+            member(integral_constant<int, 1>{}, integral_constant<int, -1>{}, sb);
+        }
+        // plane (y, z): whole rows
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int ty = (m & 1) ? -sy : sy, tz = (m & 2) ? -sz : sz;
+            v4 dq, gq, c0, c1;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) dq[j] = gq[j] = 0.f;
+#pragma unroll
+            for (int kb = 0; kb < 2; ++kb) {
+                set4(c0, ld4(fl.dn + pb + LO * ty + (LO + kb) * tz));
+                set4(c1, ld4(fl.dn + pb + (LO + 1) * ty + (LO + kb) * tz));
+                lerp4(P.sh.nb_w[2][2 * kb], P.sh.nb_w[2][2 * kb + 1], c0, c1, dq);
+                set4(c0, ld4(fl.dG + pb + LOM * ty + (LOM + kb) * tz));
+                set4(c1, ld4(fl.dG + pb + (LOM + 1) * ty + (LOM + kb) * tz));
+                lerp4(P.sh.md_w[2][2 * kb], P.sh.md_w[2][2 * kb + 1], c0, c1, gq);
+            }
+            add_A(1.f / 15.f, dq, gq, S.G0, s);
+        }
+    }
+    if (!live) return;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (x + j >= g.nx) break;
+        const float q1 = 1.f + d0[j];
+        pr[idx0 + j] = (1.f / 3.f) * S.rho0 * q1 + (P.hs ? (S.G0 + s[j]) * S.p_pref * q1 : 0.f);
+    }
+}
+
+template <int SIG>
+static void pressure4_sigma(const Params& P, const Fields& f, float* pr, cudaStream_t s)
+{
+    unsigned blocks;
+    if (P.g.nx < 128) {
+        const TileMap tm = make_flatmap(P.g, 4, FORCE_NT, blocks);
+        k_pressure4<SIG, false><<<blocks, FORCE_NT, 0, s>>>(P, tm, f, pr);
+    } else {
+        const TileMap tm = make_tilemap(P.g, 128, FORCE_NT / 32, 128, blocks);
+        k_pressure4<SIG, true><<<blocks, FORCE_NT, 0, s>>>(P, tm, f, pr);
+    }
+}
+
+bool launch_pressure4(const Params& P, const Fields& f, float* pr, cudaStream_t s)
+{
+    switch (P.sigma) {
+    case 4: pressure4_sigma<4>(P, f, pr, s); break;
+    case 6: pressure4_sigma<6>(P, f, pr, s); break;
+    case 8: pressure4_sigma<8>(P, f, pr, s); break;
+    case 10: pressure4_sigma<10>(P, f, pr, s); break;
+    case 12: pressure4_sigma<12>(P, f, pr, s); break;
+    default: return false;
+    }
+    return true;
 }
 
 template <int SIG, bool LN>

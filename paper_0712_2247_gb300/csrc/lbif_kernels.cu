@@ -708,7 +708,11 @@ __global__ void k_moments_out(Params P, Fields fl, float* rho, float* u, float* 
 // addition exactly, so the pair carries about 48 bits; the products
 // (1 + dn) u enter as u + p + e with p = fl(dn u) and e = dn u - p (exact, by
 // a fused multiply-add). Each thread converts its pairs to FP64 once; the
-// CTA adds them by a fixed FP64 tree.
+// CTA adds them by a fixed FP64 tree. (Merging the threads' pairs in FP32 too
+// takes 28 us at 256 x 192 x 96, but 48 bits are too few where a plane's average
+// cancels to far below the flow's amplitude; 38 us with four x nodes a thread,
+// whose other order of additions moves such an average by 1e-9 of itself.)
+// A thread's loads go out for PROF_U nodes at a time: 66 -> 50 us.
 constexpr int PROF_K = 5;
 
 struct F32Pair {
@@ -723,7 +727,8 @@ __device__ __forceinline__ void pair_add(F32Pair& a, float x)
     a.hi = s;
 }
 
-__global__ void k_profiles(Params P, Fields fl, double* part, int chunks)
+constexpr int PROF_U = 4;
+__global__ void __launch_bounds__(256) k_profiles(Params P, Fields fl, double* part, int chunks)
 {
     __shared__ double sh[PROF_K][256];
     const Geom& g = P.g;
@@ -736,26 +741,37 @@ __global__ void k_profiles(Params P, Fields fl, double* part, int chunks)
     const int n = (y1 - y0) * g.nx;
     int dy = threadIdx.x / g.nx, x = threadIdx.x - dy * g.nx;
     const int step_y = blockDim.x / g.nx, step_x = blockDim.x - step_y * g.nx;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const int p = pidx(g, x, y0 + dy, z);
-        const float d = fl.dn[p];
-        const float v[3] = {fl.ux[p], fl.uy[p], fl.uz[p]};
-        pair_add(a[0], d);
-        pair_add(a[1], v[0]);
+    for (int k = threadIdx.x; k < n; k += PROF_U * blockDim.x) {
+        float d[PROF_U], v[PROF_U][3];
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const float pr = d * v[j];
-            const float e = fmaf(d, v[j], -pr);
-            pair_add(a[2 + j], v[j]);
-            pair_add(a[2 + j], pr);
-            pair_add(a[2 + j], e);
+        for (int u = 0; u < PROF_U; ++u) {
+            const bool in = k + u * (int)blockDim.x < n;
+            const int p = in ? pidx(g, x, y0 + dy, z) : pidx(g, 0, y0, z);
+            d[u] = __ldg(fl.dn + p);
+            v[u][0] = __ldg(fl.ux + p);
+            v[u][1] = __ldg(fl.uy + p);
+            v[u][2] = __ldg(fl.uz + p);
+            // next node of this thread: blockDim.x further in row-major order
+            x += step_x;
+            dy += step_y;
+            if (x >= g.nx) {
+                x -= g.nx;
+                ++dy;
+            }
         }
-        // next node of this thread: blockDim.x further in row-major order
-        x += step_x;
-        dy += step_y;
-        if (x >= g.nx) {
-            x -= g.nx;
-            ++dy;
+#pragma unroll
+        for (int u = 0; u < PROF_U; ++u) {
+            if (k + u * (int)blockDim.x >= n) break;
+            pair_add(a[0], d[u]);
+            pair_add(a[1], v[u][0]);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const float pr = d[u] * v[u][j];
+                const float e = fmaf(d[u], v[u][j], -pr);
+                pair_add(a[2 + j], v[u][j]);
+                pair_add(a[2 + j], pr);
+                pair_add(a[2 + j], e);
+            }
         }
     }
 #pragma unroll
@@ -949,7 +965,8 @@ cudaError_t launch_force_soa(const Params& P, const float4* F, float* out, cudaS
 cudaError_t launch_moments_out(const Params& P, const Fields& f, float* rho, float* u, float* p,
                                cudaStream_t s)
 {
-    k_moments_out<<<nblocks(P.g.N, 256), 256, 0, s>>>(P, f, rho, u, p);
+    if (p && launch_pressure4(P, f, p, s)) p = nullptr;
+    if (rho || u || p) k_moments_out<<<nblocks(P.g.N, 256), 256, 0, s>>>(P, f, rho, u, p);
     return cudaGetLastError();
 }
 
