@@ -488,10 +488,14 @@ __global__ void __launch_bounds__(BALL_THREADS) k_ball_tma(Params P, const __gri
     }
 }
 
-// Narrow grids (a 32 x 8 tile would leave most lanes idle): one thread per
+// Narrow grids (a 32 x 16 tile would leave most lanes idle): one thread per
 // node, reading the padded field directly. The additions run in the order of
 // k_ball (row sums grown outwards from the centre, disc sums over y, then the
-// planes in increasing z), so both kernels give bit-identical results.
+// planes in increasing z), so both kernels give bit-identical results. Radii up
+// to 4 are unrolled, so that a node's loads (33 at R = 2, 257 at R = 4) go out
+// together instead of one chain of a few at a time: at R = 2, 2048 slits of 4 x 4
+// 57 -> 30 us, 16 x 16 x 32 13 -> 7.4 us.
+template <int R0>
 __global__ void __launch_bounds__(256) k_ball_direct(Params P, const float* __restrict__ dn,
                                                      float* __restrict__ dG, int* status, int skip_done)
 {
@@ -501,21 +505,42 @@ __global__ void __launch_bounds__(256) k_ball_direct(Params P, const float* __re
     decompose(P.g, idx, x, y, z);
     const int so = slit_of(P, z);
     if (so < 0 || (skip_done && frozen(P, so))) return;
-    const int R = P.sigma / 2;
     const int p = pidx(P.g, x, y, z);
+    const int sy = P.g.px, sz = P.g.px * P.g.py;
     float s = 0.f;
-    for (int dz = -R; dz <= R; ++dz) {
-        float D = 0.f;
-        for (int dy = -R; dy <= R; ++dy) {
-            const int rem = R * R - dy * dy - dz * dz;
-            if (rem < 0) continue;
-            const int w = cisqrt(rem);
-            const float* row = dn + p + (dz * P.g.py + dy) * P.g.px;
-            float r = __ldg(row);
-            for (int dx = 1; dx <= w; ++dx) r += __ldg(row - dx) + __ldg(row + dx);
-            D += r;
+    if constexpr (R0 > 0) {
+#pragma unroll
+        for (int dz = -R0; dz <= R0; ++dz) {
+            float D = 0.f;
+#pragma unroll
+            for (int dy = -R0; dy <= R0; ++dy) {
+                const int rem = R0 * R0 - dy * dy - dz * dz;
+                if (rem < 0) continue;
+                const int w = cisqrt(rem);
+                const float* row = dn + p + (dz * sz + dy * sy);
+                float r = __ldg(row);
+#pragma unroll
+                for (int dx = 1; dx <= R0; ++dx)
+                    if (dx <= w) r += __ldg(row - dx) + __ldg(row + dx);
+                D += r;
+            }
+            s += D;
         }
-        s += D;
+    } else {
+        const int R = P.sigma / 2;
+        for (int dz = -R; dz <= R; ++dz) {
+            float D = 0.f;
+            for (int dy = -R; dy <= R; ++dy) {
+                const int rem = R * R - dy * dy - dz * dz;
+                if (rem < 0) continue;
+                const int w = cisqrt(rem);
+                const float* row = dn + p + (dz * sz + dy * sy);
+                float r = __ldg(row);
+                for (int dx = 1; dx <= w; ++dx) r += __ldg(row - dx) + __ldg(row + dx);
+                D += r;
+            }
+            s += D;
+        }
     }
     bool bad;
     float v = g2_deviation(P, P.sl[so].eta0, s * P.ball_inv, bad);
@@ -921,8 +946,20 @@ void ball_box(int sigma, int* W, int* H)
 cudaError_t launch_ball(const Params& P, const float* dn, float* dG, int* status, int want,
                         int skip_done, cudaStream_t s, const CUtensorMap* tmap)
 {
-    if (P.g.nx < BALL_TX / 2 || P.g.ny < BALL_TY / 2) {
-        k_ball_direct<<<nblocks(P.g.N, 256), 256, 0, s>>>(P, dn, dG, status, skip_done);
+    // direct sums below half a tile, and for the two smallest radii below a whole
+    // tile row (20 x 200 x 150, sigma 4: tiles 18, direct 14 us; 128 slits of 32 x 32:
+    // tiles 58, direct 72 us)
+    if (P.g.nx < (P.sigma <= 4 ? BALL_TX : BALL_TX / 2) || P.g.ny < BALL_TY / 2) {
+        // small blocks on small grids, so that the SMs share them
+        const int nt = P.g.N < 256LL * NUM_SMS ? 64 : 256;
+        const unsigned nb = nblocks(P.g.N, nt);
+        switch (P.sigma / 2) {
+        case 1: k_ball_direct<1><<<nb, nt, 0, s>>>(P, dn, dG, status, skip_done); break;
+        case 2: k_ball_direct<2><<<nb, nt, 0, s>>>(P, dn, dG, status, skip_done); break;
+        case 3: k_ball_direct<3><<<nb, nt, 0, s>>>(P, dn, dG, status, skip_done); break;
+        case 4: k_ball_direct<4><<<nb, nt, 0, s>>>(P, dn, dG, status, skip_done); break;
+        default: k_ball_direct<0><<<nb, nt, 0, s>>>(P, dn, dG, status, skip_done); break;
+        }
         return cudaGetLastError();
     }
     switch (P.sigma / 2) {
