@@ -169,6 +169,7 @@ __device__ __forceinline__ void node_force(const Params& P, const SlitParam& S, 
 __global__ void __launch_bounds__(256) k_force(Params P, TileMap tm, Fields fl,
                                                const float4* __restrict__ Ft, float4* __restrict__ F)
 {
+    step_begin(P);
     const Geom& g = P.g;
     int x, y, z;
     if (tm.flat) {
@@ -557,6 +558,7 @@ template <int SIG, bool C2, bool LN>
 __global__ void __launch_bounds__(FORCE_NT, FORCE_MINB) k_force4(Params P, TileMap tm, Fields fl,
                                                 const float4* __restrict__ Ft, float4* __restrict__ F)
 {
+    step_begin(P);
     const Geom& g = P.g;
     int x, y, z;
     bool live = true;
@@ -771,25 +773,23 @@ bool launch_pressure4(const Params& P, const Fields& f, float* pr, cudaStream_t 
 }
 
 template <int SIG, bool LN>
-static void force4_launch(const Params& P, const TileMap& tm, const Fields& f, const float4* Ft, float4* F,
+static cudaError_t force4_launch(const Params& P, const TileMap& tm, const Fields& f, const float4* Ft, float4* F,
                           unsigned blocks, cudaStream_t s)
 {
-    if (P.c2)
-        k_force4<SIG, true, LN><<<blocks, FORCE_NT, 0, s>>>(P, tm, f, Ft, F);
-    else
-        k_force4<SIG, false, LN><<<blocks, FORCE_NT, 0, s>>>(P, tm, f, Ft, F);
+    return launch_step(P.c2 ? k_force4<SIG, true, LN> : k_force4<SIG, false, LN>, blocks, FORCE_NT, 0, s, P, tm, f, Ft,
+                       F);
 }
 
 template <int SIG>
-static void force4_sigma(const Params& P, const Fields& f, const float4* Ft, float4* F, int group, cudaStream_t s)
+static cudaError_t force4_sigma(const Params& P, const Fields& f, const float4* Ft, float4* F, int group, cudaStream_t s)
 {
     unsigned blocks;
     if (P.g.nx < 128) {
         const TileMap tm = make_flatmap(P.g, 4, FORCE_NT, blocks);
-        force4_launch<SIG, false>(P, tm, f, Ft, F, blocks, s);
+        return force4_launch<SIG, false>(P, tm, f, Ft, F, blocks, s);
     } else {
         const TileMap tm = make_tilemap(P.g, 128, FORCE_NT / 32, group, blocks);
-        force4_launch<SIG, true>(P, tm, f, Ft, F, blocks, s);
+        return force4_launch<SIG, true>(P, tm, f, Ft, F, blocks, s);
     }
 }
 
@@ -802,18 +802,17 @@ cudaError_t launch_force(const Params& P, const Fields& f, const float4* Ft, flo
 {
     if (group <= 0) group = 128;
     switch (P.sigma) {
-    case 4: force4_sigma<4>(P, f, Ft, F, group, s); break;
-    case 6: force4_sigma<6>(P, f, Ft, F, group, s); break;
-    case 8: force4_sigma<8>(P, f, Ft, F, group, s); break;
-    case 10: force4_sigma<10>(P, f, Ft, F, group, s); break;
-    case 12: force4_sigma<12>(P, f, Ft, F, group, s); break;
+    case 4: return force4_sigma<4>(P, f, Ft, F, group, s);
+    case 6: return force4_sigma<6>(P, f, Ft, F, group, s);
+    case 8: return force4_sigma<8>(P, f, Ft, F, group, s);
+    case 10: return force4_sigma<10>(P, f, Ft, F, group, s);
+    case 12: return force4_sigma<12>(P, f, Ft, F, group, s);
     default: {
         unsigned blocks;
         const TileMap tm = P.g.nx < 32 ? make_flatmap(P.g, 1, 256, blocks) : make_tilemap(P.g, 32, 8, group, blocks);
-        k_force<<<blocks, 256, 0, s>>>(P, tm, f, Ft, F);
+        return launch_step(k_force, blocks, 256, 0, s, P, tm, f, Ft, F);
     }
     }
-    return cudaGetLastError();
 }
 
 }  // namespace lbif

@@ -106,6 +106,7 @@ __global__ void k_init_profiles(Params P, float* dn, float* ux, float* uy, float
 
 __global__ void k_tick(Params P, int4* clk)
 {
+    step_begin(P);
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= P.nslits || frozen(P, s)) return;
     int4 c = clk[s];
@@ -372,6 +373,7 @@ __global__ void __launch_bounds__(BALL_THREADS) k_ball(Params P, const float* __
                                               float* __restrict__ dG, int* status, int zchunk,
                                               int skip_done)
 {
+    step_begin(P);
     constexpr int TX = BALL_TX, TY = BALL_TY;
     constexpr int C4 = ball_c4<R>();
     constexpr int W = TX + 2 * C4, H = TY + 2 * R;
@@ -418,6 +420,7 @@ __global__ void __launch_bounds__(BALL_THREADS) k_ball_tma(Params P, const __gri
                                                   float* __restrict__ dG, int* status, int zchunk,
                                                   int skip_done)
 {
+    step_begin(P);
     constexpr int TX = BALL_TX, TY = BALL_TY;
     constexpr int C4 = ball_c4<R>();
     constexpr int W = TX + 2 * C4, H = TY + 2 * R;
@@ -499,6 +502,7 @@ template <int R0>
 __global__ void __launch_bounds__(256) k_ball_direct(Params P, const float* __restrict__ dn,
                                                      float* __restrict__ dG, int* status, int skip_done)
 {
+    step_begin(P);
     long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (idx >= P.g.N) return;
     int x, y, z;
@@ -862,8 +866,7 @@ cudaError_t launch_init_fields(const Params& P, float* const f[4], const float* 
 
 cudaError_t launch_tick(const Params& P, int4* clk, cudaStream_t s)
 {
-    k_tick<<<nblocks(P.nslits, 128), 128, 0, s>>>(P, clk);
-    return cudaGetLastError();
+    return launch_step(k_tick, nblocks(P.nslits, 128), 128, 0, s, P, clk);
 }
 
 cudaError_t launch_pop_canon(const Params& P, void* pop, int i, void* canon, int to_pop, cudaStream_t s)
@@ -930,10 +933,9 @@ static cudaError_t ball_r(const Params& P, const float* dn, float* dG, int* stat
     nchunk = (g.nz + zchunk - 1) / zchunk;
     dim3 grid(gx, gy, nchunk);
     if (tmap)
-        k_ball_tma<R><<<grid, BALL_THREADS, smem, s>>>(P, *tmap, dG, status, zchunk, skip_done);
+        return launch_step(k_ball_tma<R>, grid, BALL_THREADS, smem, s, P, *tmap, dG, status, zchunk, skip_done);
     else
-        k_ball<R><<<grid, BALL_THREADS, smem, s>>>(P, dn, dG, status, zchunk, skip_done);
-    return cudaGetLastError();
+        return launch_step(k_ball<R>, grid, BALL_THREADS, smem, s, P, dn, dG, status, zchunk, skip_done);
 }
 
 void ball_box(int sigma, int* W, int* H)
@@ -954,11 +956,11 @@ cudaError_t launch_ball(const Params& P, const float* dn, float* dG, int* status
         const int nt = P.g.N < 256LL * NUM_SMS ? 64 : 256;
         const unsigned nb = nblocks(P.g.N, nt);
         switch (P.sigma / 2) {
-        case 1: k_ball_direct<1><<<nb, nt, 0, s>>>(P, dn, dG, status, skip_done); break;
-        case 2: k_ball_direct<2><<<nb, nt, 0, s>>>(P, dn, dG, status, skip_done); break;
-        case 3: k_ball_direct<3><<<nb, nt, 0, s>>>(P, dn, dG, status, skip_done); break;
-        case 4: k_ball_direct<4><<<nb, nt, 0, s>>>(P, dn, dG, status, skip_done); break;
-        default: k_ball_direct<0><<<nb, nt, 0, s>>>(P, dn, dG, status, skip_done); break;
+        case 1: return launch_step(k_ball_direct<1>, nb, nt, 0, s, P, dn, dG, status, skip_done);
+        case 2: return launch_step(k_ball_direct<2>, nb, nt, 0, s, P, dn, dG, status, skip_done);
+        case 3: return launch_step(k_ball_direct<3>, nb, nt, 0, s, P, dn, dG, status, skip_done);
+        case 4: return launch_step(k_ball_direct<4>, nb, nt, 0, s, P, dn, dG, status, skip_done);
+        default: return launch_step(k_ball_direct<0>, nb, nt, 0, s, P, dn, dG, status, skip_done);
         }
         return cudaGetLastError();
     }

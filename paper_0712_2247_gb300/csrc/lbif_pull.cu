@@ -724,6 +724,7 @@ __global__ void __launch_bounds__(CSM_THREADS, PAIR_MINB)
     k_pull_pair(Params P, PullPtrs pp, CsmIO io, const float4* __restrict__ F, int lz, int tiles_x, int tiles_y,
                 int* status)
 {
+    step_begin(P);
     constexpr int NT = CSM_THREADS, TY = NT / TX, HX = TX + 2;
     constexpr bool RAW = F16_RAW<T>;
     extern __shared__ __align__(16) float2 psm[];
@@ -1128,6 +1129,7 @@ template <typename T, bool IP>
 __global__ void __launch_bounds__(BLOCK_NT) k_pull_block(Params P, const T* pin, T* pout, CsmIO io,
                                                          const float4* __restrict__ F, int tz, int* status)
 {
+    step_begin(P);
     __shared__ float st[CSM_NF * BLOCK_NS];
     constexpr bool RAW = F16_RAW<T>;
     const Geom& g = P.g;
@@ -1191,8 +1193,8 @@ static cudaError_t pull_block(const Params& P, const void* pin, void* pout, cons
     const int share = (g.nz + 2 * NUM_SMS - 1) / (2 * NUM_SMS);
     if (tz > share) tz = share;
     const int threads = (tz * A + 31) / 32 * 32;
-    k_pull_block<T, IP><<<(g.nz + tz - 1) / tz, threads, 0, s>>>(P, (const T*)pin, (T*)pout, io, F, tz, status);
-    return cudaGetLastError();
+    return launch_step(k_pull_block<T, IP>, (g.nz + tz - 1) / tz, threads, 0, s, P, (const T*)pin, (T*)pout, io, F, tz,
+                       status);
 }
 
 bool csm_ok(const Geom& g) { return g.nx >= CSM_TX && g.ny >= CSM_TY; }
@@ -1251,8 +1253,7 @@ static cudaError_t pull_pair(const Params& P, const void* pin, void* pout, const
         pp.src[i] = static_cast<const T*>(pin) + P.dbase[i] + back;
         pp.dst[i] = static_cast<T*>(pout) + P.dbase[i];
     }
-    k_pull_pair<T, IP, TX><<<(unsigned)blocks, CSM_THREADS, smem, s>>>(P, pp, io, F, lz, tx, ty, status);
-    return cudaGetLastError();
+    return launch_step(k_pull_pair<T, IP, TX>, (unsigned)blocks, CSM_THREADS, smem, s, P, pp, io, F, lz, tx, ty, status);
 }
 
 // The tile's width: the one that covers the cross-section with the least work,
