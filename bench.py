@@ -113,11 +113,11 @@ def kernel_bytes(storage: int):
 
 # DRAM bytes per node of each step kernel (dram__bytes_read.sum + dram__bytes_write.sum of one
 # ncu capture on the 128x128x192 sigma = 12 slit, default launch shapes, divided by its nodes;
-# the same per-node traffic as the 256x256x192 capture of the pull pass, so it scales with the
-# nodes of a launch). The ball kernel's dG writes stay in L2 at that size: read bytes only.
-TRAFFIC_B_PER_NODE = {0: {"ball_g2": 5.8, "force": 40.9, "collide_stream": 209.7},
-                      1: {"ball_g2": 5.8, "force": 40.9, "collide_stream": 157.5}}
-# the in-place pull pass (FP32; the FP16 in-place populations of that capture,
+# the pull pass: a 256x128x192 capture of k_pull_pair; the traffic scales with the nodes of a
+# launch). The ball kernel's dG writes stay in L2 at that size: read bytes only.
+TRAFFIC_B_PER_NODE = {0: {"ball_g2": 5.8, "force": 40.9, "collide_stream": 202.7},
+                      1: {"ball_g2": 5.8, "force": 40.9, "collide_stream": 126.9}}
+# the in-place pull pass (FP32, captured with the one-plane form, which moves the same lines; the FP16 in-place populations of that capture,
 # 120 MB, nearly fit in L2, so its DRAM figure does not scale and is left out)
 TRAFFIC_INPLACE = {0: {"ball_g2": 5.8, "force": 40.9, "collide_stream": 197.1}}
 
