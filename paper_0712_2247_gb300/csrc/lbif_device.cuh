@@ -34,8 +34,13 @@ __device__ __forceinline__ constexpr float kW(int i)
 __device__ __forceinline__ constexpr int kC2(int i) { return kCx(i) * kCx(i) + kCy(i) * kCy(i) + kCz(i) * kCz(i); }
 __device__ __forceinline__ constexpr int opp_of(int i) { return i == 0 ? 0 : ((i & 1) ? i + 1 : i - 1); }
 
-__device__ __forceinline__ float ldp(const float* p) { return __ldg(p); }
-__device__ __forceinline__ float ldp(const __half* p) { return __half2float(__ldg(p)); }
+// Loads of what the step's kernels write (fields, forces, populations, clocks).
+// Ordinary ones: a kernel under programmatic launch (step_begin) runs while its
+// predecessor still writes them, where a read-only load (__ldg, or one that the
+// compiler makes of a const __restrict__ argument) has no defined value. __ldg is
+// for the tables that no kernel of a step writes.
+__device__ __forceinline__ float ldp(const float* p) { return *p; }
+__device__ __forceinline__ float ldp(const __half* p) { return __half2float(*p); }
 // RAW: a 16-bit population is kept as its bits in the float's register and
 // converted at its first use (late_cvt), so that no instruction waits on the
 // gather before the work that is meant to hide its latency
@@ -45,14 +50,14 @@ template <bool RAW>
 __device__ __forceinline__ float ldq(const __half* p)
 {
     if constexpr (RAW)
-        return __int_as_float((int)__half_as_ushort(__ldg(p)));
+        return __int_as_float((int)__half_as_ushort(*p));
     else
         return ldp(p);
 }
 __device__ __forceinline__ float late_cvt(float bits) { return __half2float(__ushort_as_half((unsigned short)__float_as_int(bits))); }
 __device__ __forceinline__ void stp(float* p, float v) { *p = v; }
 __device__ __forceinline__ void stp(__half* p, float v) { *p = __float2half_rn(v); }
-__device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
 __device__ __forceinline__ int pidx(const Geom& g, int x, int y, int z)
 {
@@ -269,7 +274,7 @@ struct IpSlots {
 
 __device__ __forceinline__ IpSlots ip_slots(const Params& P, const SlitParam& S, int s, int x, int y, int z)
 {
-    const int4 c = __ldg(P.clk + s);
+    const int4 c = P.clk[s];
     IpSlots q;
     q.nx = P.g.nx;
     q.ny = P.g.ny;
@@ -296,7 +301,8 @@ __device__ __forceinline__ IpSlots ip_slots(const Params& P, const SlitParam& S,
 // its predecessor still runs. Every thread of such a kernel calls step_begin()
 // first: it waits for the predecessor's end (and so, every kernel of the chain
 // doing the same, for all earlier work) before it reads or writes anything, then
-// lets the successor come up.
+// lets the successor come up. What it reads of its predecessors goes through
+// ordinary loads (ldp).
 //
 // The attribute is given up to 512 nodes per SM. Microseconds per step without /
 // with it at sigma 4 and 10: 8 x 8 x 16 20.8 / 16.5 and 50.5 / 48.1, 16 x 16 x 32

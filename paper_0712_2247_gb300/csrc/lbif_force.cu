@@ -28,9 +28,9 @@ __device__ __forceinline__ void axis_pair(const Params& P, const Fields& fl, int
 {
     const int o = P.sh.ax_nb[A], om = P.sh.ax_md[A];
     const float* uf = ufield<A>(fl);
-    float dp = __ldg(fl.dn + p + o), dm = __ldg(fl.dn + p - o);
-    float up = __ldg(uf + p + o), um = __ldg(uf + p - o);
-    float gp = __ldg(fl.dG + p + om), gm = __ldg(fl.dG + p - om);
+    float dp = ldp(fl.dn + p + o), dm = ldp(fl.dn + p - o);
+    float up = ldp(uf + p + o), um = ldp(uf + p - o);
+    float gp = ldp(fl.dG + p + om), gm = ldp(fl.dG + p - om);
     float Ap = shell_A(dp, gp, G0), Am = shell_A(dm, gm, G0);
     const float DA = A == 2 ? Ap - Am : fmaf(G0, dp - dm, fmaf(gp - gm, 1.f + dp, gm * (dp - dm)));
     f[A] += (1.f / 30.f) * (DA - lk * ((G0 + Ap) * (up - u0[A]) - (G0 + Am) * (u0[A] - um)));
@@ -52,7 +52,7 @@ __device__ __forceinline__ void diag_quartet(const Params& P, const Fields& fl, 
     auto md = [&](int m, int k) { return p + ((m & 1) ? -1 : 1) * P.sh.md_a[PL][k] + ((m & 2) ? -1 : 1) * P.sh.md_b[PL][k]; };
     if constexpr (PL == 0) {
         // relative to the node's own n and g2: every member a small deviation
-        const float d0 = __ldg(fl.dn + p), g0 = __ldg(fl.dG + p);
+        const float d0 = ldp(fl.dn + p), g0 = ldp(fl.dG + p);
         const float Aref = fmaf(G0, d0, g0 * (1.f + d0));
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
@@ -61,10 +61,10 @@ __device__ __forceinline__ void diag_quartet(const Params& P, const Fields& fl, 
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const float w = P.sh.nb_w[PL][k], wm = P.sh.md_w[PL][k];
-                dl = fmaf(w, __ldg(fl.dn + nb(m, k)) - d0, dl);
-                ua = fmaf(w, __ldg(fa + nb(m, k)), ua);
-                ub = fmaf(w, __ldg(fb + nb(m, k)), ub);
-                gl = fmaf(wm, __ldg(fl.dG + md(m, k)) - g0, gl);
+                dl = fmaf(w, ldp(fl.dn + nb(m, k)) - d0, dl);
+                ua = fmaf(w, ldp(fa + nb(m, k)), ua);
+                ub = fmaf(w, ldp(fb + nb(m, k)), ub);
+                gl = fmaf(wm, ldp(fl.dG + md(m, k)) - g0, gl);
             }
             const float av = fmaf(G0 + g0, dl, gl * ((1.f + d0) + dl));
             const float GA = G0 + (Aref + av);
@@ -88,9 +88,9 @@ __device__ __forceinline__ void diag_quartet(const Params& P, const Fields& fl, 
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const float w = P.sh.nb_w[PL][k], wm = P.sh.md_w[PL][k];
-            const float n1 = __ldg(fl.dn + nb(m, k)), n2 = __ldg(fl.dn + nb(mp, k));
-            const float b1 = __ldg(fb + nb(m, k)), b2 = __ldg(fb + nb(mp, k));
-            const float g1 = __ldg(fl.dG + md(m, k)), g2 = __ldg(fl.dG + md(mp, k));
+            const float n1 = ldp(fl.dn + nb(m, k)), n2 = ldp(fl.dn + nb(mp, k));
+            const float b1 = ldp(fb + nb(m, k)), b2 = ldp(fb + nb(mp, k));
+            const float g1 = ldp(fl.dG + md(m, k)), g2 = ldp(fl.dG + md(mp, k));
             dm = fmaf(w, n1, dm);
             dpp = fmaf(w, n2, dpp);
             Dd = fmaf(w, n1 - n2, Dd);
@@ -100,8 +100,8 @@ __device__ __forceinline__ void diag_quartet(const Params& P, const Fields& fl, 
             gm = fmaf(wm, g1, gm);
             gp = fmaf(wm, g2, gp);
             Dg = fmaf(wm, g1 - g2, Dg);
-            am = fmaf(w, __ldg(fa + nb(m, k)), am);
-            ap = fmaf(w, __ldg(fa + nb(mp, k)), ap);
+            am = fmaf(w, ldp(fa + nb(m, k)), am);
+            ap = fmaf(w, ldp(fa + nb(mp, k)), ap);
         }
         const float Am = shell_A(dm, gm, G0), Ap = shell_A(dpp, gp, G0);
         const float DA = fmaf(G0, Dd, fmaf(Dg, 1.f + dm, gp * Dd));
@@ -129,11 +129,11 @@ __device__ __forceinline__ float coupling_factor(const Params& P, const SlitPara
 // total force F / n0 at a node (body + hard sphere + tail), and the energy
 // source of Eq. C2eq over n0 when it is on (0 otherwise)
 __device__ __forceinline__ void node_force(const Params& P, const SlitParam& S, const Fields& fl,
-                                           const float4* __restrict__ Ft, long long idx, int z,
+                                           const float4* Ft, long long idx, int z,
                                            int p, float& fx, float& fy, float& fz, float& c2)
 {
-    const float d0 = __ldg(fl.dn + p);
-    const float u0[3] = {__ldg(fl.ux + p), __ldg(fl.uy + p), __ldg(fl.uz + p)};
+    const float d0 = ldp(fl.dn + p);
+    const float u0[3] = {ldp(fl.ux + p), ldp(fl.uy + p), ldp(fl.uz + p)};
     float opd = 1.f + d0;
     fx = opd * S.body[0];
     fy = opd * S.body[1];
@@ -167,7 +167,7 @@ __device__ __forceinline__ void node_force(const Params& P, const SlitParam& S, 
 }
 
 __global__ void __launch_bounds__(256) k_force(Params P, TileMap tm, Fields fl,
-                                               const float4* __restrict__ Ft, float4* __restrict__ F)
+                                               const float4* Ft, float4* __restrict__ F)
 {
     step_begin(P);
     const Geom& g = P.g;
@@ -222,7 +222,7 @@ __device__ __forceinline__ float2 shell_A2(float2 dq, float2 gq, float G0)
 
 // values at x offsets D..D+3 of a float4-aligned base
 template <int D>
-__device__ __forceinline__ void win(const float* __restrict__ f, int b, v4 r)
+__device__ __forceinline__ void win(const float* f, int b, v4 r)
 {
     constexpr int B4 = floor4(D), RR = D - B4;
     if constexpr (RR == 0) {
@@ -248,14 +248,14 @@ struct Lanes {
 // window costs the float4's wavefronts only (a strided scalar load costs as
 // many again).
 template <int D, bool LN>
-__device__ __forceinline__ void win2(const float* __restrict__ f, int b, v4 w0, v4 w1, Lanes ln)
+__device__ __forceinline__ void win2(const float* f, int b, v4 w0, v4 w1, Lanes ln)
 {
     constexpr int RR = D - floor4(D);
     if constexpr (RR == 0) {
         const float4 A = ld4(f + b + D);
         float s = 0.f;
         if constexpr (LN) s = __shfl_down_sync(0xffffffffu, A.x, 1);
-        if (!LN || ln.hi) s = __ldg(f + b + D + 4);
+        if (!LN || ln.hi) s = ldp(f + b + D + 4);
         set4(w0, A);
         w1[0] = A.y;
         w1[1] = A.z;
@@ -265,7 +265,7 @@ __device__ __forceinline__ void win2(const float* __restrict__ f, int b, v4 w0, 
         const float4 C = ld4(f + b + D + 1);
         float s = 0.f;
         if constexpr (LN) s = __shfl_up_sync(0xffffffffu, C.w, 1);
-        if (!LN || ln.lo) s = __ldg(f + b + D);
+        if (!LN || ln.lo) s = ldp(f + b + D);
         w0[0] = s;
         w0[1] = C.x;
         w0[2] = C.y;
@@ -285,7 +285,7 @@ __device__ __forceinline__ void win2(const float* __restrict__ f, int b, v4 w0, 
 // x offsets of the two corners of a member with x sign SA: SA > 0: (LO, LO+1),
 // SA < 0: (-LO, -LO-1); returns the windows in corner order (ka = 0, 1)
 template <int LO, int SA, bool LN>
-__device__ __forceinline__ void corners_x(const float* __restrict__ f, int b, v4 c0, v4 c1, Lanes ln)
+__device__ __forceinline__ void corners_x(const float* f, int b, v4 c0, v4 c1, Lanes ln)
 {
     if constexpr (SA > 0)
         win2<LO, LN>(f, b, c0, c1, ln);
@@ -556,7 +556,7 @@ constexpr int FORCE_NT = 64;
 #endif
 template <int SIG, bool C2, bool LN>
 __global__ void __launch_bounds__(FORCE_NT, FORCE_MINB) k_force4(Params P, TileMap tm, Fields fl,
-                                                const float4* __restrict__ Ft, float4* __restrict__ F)
+                                                const float4* Ft, float4* __restrict__ F)
 {
     step_begin(P);
     const Geom& g = P.g;

@@ -369,7 +369,7 @@ __device__ __forceinline__ void ball_disc_out(const Params& P, const float* __re
 // them into a register ring of the 2R+1 output planes they touch, emit the
 // completed plane.
 template <int R>
-__global__ void __launch_bounds__(BALL_THREADS) k_ball(Params P, const float* __restrict__ dn,
+__global__ void __launch_bounds__(BALL_THREADS) k_ball(Params P, const float* dn,
                                               float* __restrict__ dG, int* status, int zchunk,
                                               int skip_done)
 {
@@ -457,6 +457,9 @@ __global__ void __launch_bounds__(BALL_THREADS) k_ball_tma(Params P, const __gri
             : "memory");
     };
     if (threadIdx.x == 0) {
+        // the density was written by ordinary stores of a kernel that step_begin
+        // waited for, not by an earlier launch boundary: order the copies after them
+        asm volatile("fence.proxy.async.global;" ::: "memory");
         issue(0);
         if (np > 1) issue(1);
     }
@@ -499,7 +502,7 @@ __global__ void __launch_bounds__(BALL_THREADS) k_ball_tma(Params P, const __gri
 // together instead of one chain of a few at a time: at R = 2, 2048 slits of 4 x 4
 // 57 -> 30 us, 16 x 16 x 32 13 -> 7.4 us.
 template <int R0>
-__global__ void __launch_bounds__(256) k_ball_direct(Params P, const float* __restrict__ dn,
+__global__ void __launch_bounds__(256) k_ball_direct(Params P, const float* dn,
                                                      float* __restrict__ dG, int* status, int skip_done)
 {
     step_begin(P);
@@ -522,10 +525,10 @@ __global__ void __launch_bounds__(256) k_ball_direct(Params P, const float* __re
                 if (rem < 0) continue;
                 const int w = cisqrt(rem);
                 const float* row = dn + p + (dz * sz + dy * sy);
-                float r = __ldg(row);
+                float r = ldp(row);
 #pragma unroll
                 for (int dx = 1; dx <= R0; ++dx)
-                    if (dx <= w) r += __ldg(row - dx) + __ldg(row + dx);
+                    if (dx <= w) r += ldp(row - dx) + ldp(row + dx);
                 D += r;
             }
             s += D;
@@ -539,8 +542,8 @@ __global__ void __launch_bounds__(256) k_ball_direct(Params P, const float* __re
                 if (rem < 0) continue;
                 const int w = cisqrt(rem);
                 const float* row = dn + p + (dz * sz + dy * sy);
-                float r = __ldg(row);
-                for (int dx = 1; dx <= w; ++dx) r += __ldg(row - dx) + __ldg(row + dx);
+                float r = ldp(row);
+                for (int dx = 1; dx <= w; ++dx) r += ldp(row - dx) + ldp(row + dx);
                 D += r;
             }
             s += D;

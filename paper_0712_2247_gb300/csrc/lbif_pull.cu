@@ -400,7 +400,7 @@ __device__ __forceinline__ CsmStaged csm_staged(const Geom& g, int x0, int y0)
 
 // stage plane q (-1 <= q <= nz) of the tile into `slot`
 template <int NT>
-__device__ __forceinline__ void csm_stage(const Params& P, const CsmIO& io, const float4* __restrict__ F,
+__device__ __forceinline__ void csm_stage(const Params& P, const CsmIO& io, const float4* F,
                                           float* slot, const CsmStaged& st, int q)
 {
     const Geom& g = P.g;
@@ -420,8 +420,8 @@ __device__ __forceinline__ void csm_stage(const Params& P, const CsmIO& io, cons
         if (k * NT >= CSM_HN || st.p[k] < 0) continue;
         const int h = threadIdx.x + k * NT;
         const int p = pq + st.p[k];
-        const float4 f = __ldg(Fq + st.n[k]);
-        src_terms(__ldg(io.dn + p), __ldg(io.ux + p), __ldg(io.uy + p), __ldg(io.uz + p), f.x, f.y, f.z, f.w, om,
+        const float4 f = Fq[st.n[k]];
+        src_terms(ldp(io.dn + p), ldp(io.ux + p), ldp(io.uy + p), ldp(io.uz + p), f.x, f.y, f.z, f.w, om,
                   shifted, [&](int j, float val) { slot[j * CSM_HN + h] = val; });
     }
 }
@@ -436,7 +436,7 @@ constexpr int CSM_LZ = 16;
 // wall (bounce-back: the node's own opposite population). IP: in place
 // (slots from q, see above).
 template <int I0, int I1, bool IP, typename T, bool RAW = false>
-__device__ __forceinline__ void csm_pull(const Params& P, const T* __restrict__ pin, long long idx, int x, int y,
+__device__ __forceinline__ void csm_pull(const Params& P, const T* pin, long long idx, int x, int y,
                                          int z, int zlo, int zhi, float* v, unsigned& bb, const IpSlots& q)
 {
     const Geom& g = P.g;
@@ -555,7 +555,7 @@ template <typename T>
 constexpr bool F16_RAW = sizeof(T) == 2;
 template <typename T, bool IP>
 __global__ void __launch_bounds__(CSM_THREADS, CSM_MINB)
-    k_csm(Params P, const T* pin, T* pout, CsmIO io, const float4* __restrict__ F, int lz, int tiles_x, int tiles_y,
+    k_csm(Params P, const T* pin, T* pout, CsmIO io, const float4* F, int lz, int tiles_x, int tiles_y,
           int* status)
 {
     constexpr int NT = CSM_THREADS;
@@ -721,7 +721,7 @@ struct PullPtrs {
 
 template <typename T, bool IP, int TX>
 __global__ void __launch_bounds__(CSM_THREADS, PAIR_MINB)
-    k_pull_pair(Params P, PullPtrs pp, CsmIO io, const float4* __restrict__ F, int lz, int tiles_x, int tiles_y,
+    k_pull_pair(Params P, PullPtrs pp, CsmIO io, const float4* F, int lz, int tiles_x, int tiles_y,
                 int* status)
 {
     step_begin(P);
@@ -758,18 +758,18 @@ __global__ void __launch_bounds__(CSM_THREADS, PAIR_MINB)
         const int p = (q + g.hw) * pplane + st.p[k];
         const int q0 = plane_of(q), q1 = plane_of(q + 1);
         if (q0 >= 0) {
-            a.d.x = __ldg(io.dn + p);
-            a.ux.x = __ldg(io.ux + p);
-            a.uy.x = __ldg(io.uy + p);
-            a.uz.x = __ldg(io.uz + p);
-            a.f0 = __ldg(F + (unsigned)(q0 * nxy + st.n[k]));
+            a.d.x = ldp(io.dn + p);
+            a.ux.x = ldp(io.ux + p);
+            a.uy.x = ldp(io.uy + p);
+            a.uz.x = ldp(io.uz + p);
+            a.f0 = F[(unsigned)(q0 * nxy + st.n[k])];
         }
         if (q1 >= 0) {
-            a.d.y = __ldg(io.dn + p + pplane);
-            a.ux.y = __ldg(io.ux + p + pplane);
-            a.uy.y = __ldg(io.uy + p + pplane);
-            a.uz.y = __ldg(io.uz + p + pplane);
-            a.f1 = __ldg(F + (unsigned)(q1 * nxy + st.n[k]));
+            a.d.y = ldp(io.dn + p + pplane);
+            a.ux.y = ldp(io.ux + p + pplane);
+            a.uy.y = ldp(io.uy + p + pplane);
+            a.uz.y = ldp(io.uz + p + pplane);
+            a.f1 = F[(unsigned)(q1 * nxy + st.n[k])];
         }
     };
     // planes (q, q + 1) into pair slot ab; plane q completes own slot ow, plane
@@ -992,7 +992,7 @@ void pop_box(int storage, int* W, int* H)
 template <typename T>
 __global__ void __launch_bounds__(CSM_THREADS, 4)
     k_csm_tma(Params P, const __grid_constant__ CUtensorMap pmap, const T* pin, T* pout, CsmIO io,
-              const float4* __restrict__ F, int lz, int tiles_x, int tiles_y, int* status)
+              const float4* F, int lz, int tiles_x, int tiles_y, int* status)
 {
     constexpr int NT = CSM_THREADS, XM = tma_xm<T>(), BW = tma_bw<T>(), BOX = tma_box_bytes<T>();
     constexpr int PB = tma_box_pitch<T>(), SB = Q * PB;
@@ -1127,7 +1127,7 @@ constexpr int BLOCK_A = 64, BLOCK_NT = 256, BLOCK_NS = BLOCK_NT + 2 * BLOCK_A;
 
 template <typename T, bool IP>
 __global__ void __launch_bounds__(BLOCK_NT) k_pull_block(Params P, const T* pin, T* pout, CsmIO io,
-                                                         const float4* __restrict__ F, int tz, int* status)
+                                                         const float4* F, int tz, int* status)
 {
     step_begin(P);
     __shared__ float st[CSM_NF * BLOCK_NS];
@@ -1154,8 +1154,8 @@ __global__ void __launch_bounds__(BLOCK_NT) k_pull_block(Params P, const T* pin,
         const int ks = slit_of(P, w);
         if (ks < 0 || frozen(P, ks)) continue;
         const int p = pidx(g, kx, ky, r);
-        const float4 f = __ldg(F + ((long long)w * A + kxy));
-        src_terms(__ldg(io.dn + p), __ldg(io.ux + p), __ldg(io.uy + p), __ldg(io.uz + p), f.x, f.y, f.z, f.w,
+        const float4 f = F[(long long)w * A + kxy];
+        src_terms(ldp(io.dn + p), ldp(io.ux + p), ldp(io.uy + p), ldp(io.uz + p), f.x, f.y, f.z, f.w,
                   P.sl[ks].inv_tau, shifted, [&](int j, float val) { st[j * BLOCK_NS + k] = val; });
     }
     __syncthreads();
