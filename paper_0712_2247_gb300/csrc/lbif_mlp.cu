@@ -664,29 +664,47 @@ __device__ __forceinline__ double block_sum(double s, double* sh)
     return s;
 }
 
-// A sum kept as an unevaluated FP32 pair hi + lo (about 48 bits; Knuth's
-// two-sum gives the rounding error of each addition exactly): FP64 adds and
-// conversions run at 1/64 of the FP32 rate, so a thread converts once, at the end.
-struct SumPair {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x)
-    {
-        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
-        hi = s;
+// FP64 sums of FP32 values, the thread's part x(i0), x(i0 + step), ... below n. FP64
+// adds and conversions run at 1/64 of the FP32 rate, so the sum is kept as three
+// unevaluated FP32 numbers hi + mid + lo: Knuth's two-sum gives the rounding error
+// of each addition exactly, hi's errors go to mid and mid's to lo, which leaves
+// about 72 bits where FP64 has 53. FP32 has less range: a sum that left it (or met
+// an infinity or a NaN, all of which stay in hi or mid) is done again in FP64.
+__device__ __forceinline__ float two_sum(float& a, float x)
+{
+    const float s = __fadd_rn(a, x), b = __fsub_rn(s, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, b)), __fsub_rn(x, b));
+    a = s;
+    return e;
+}
+template <class Load>
+__device__ __forceinline__ double thread_sum(long long i0, long long n, int step, Load x)
+{
+    constexpr int U = 8;  // loads that go out together
+    float hi = 0.f, mid = 0.f, lo = 0.f;
+    auto add = [&](float v) { lo = __fadd_rn(lo, two_sum(mid, two_sum(hi, v))); };
+    long long k = i0;
+    for (; k + (U - 1) * step < n; k += U * step) {
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = x(k + u * step);
+#pragma unroll
+        for (int u = 0; u < U; ++u) add(v[u]);
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
+    for (; k < n; k += step) add(x(k));
+    if (isfinite(hi) && isfinite(mid)) return (double)hi + ((double)mid + (double)lo);
+    double s = 0.0;
+    for (long long i = i0; i < n; i += step) s += (double)x(i);
+    return s;
+}
 
 // partial sums of the mask, one per block (fixed order)
 constexpr int MSUM_BLOCKS = 64;
 __global__ void __launch_bounds__(256) k_msum(const float* mask, long long n, double* part)
 {
     __shared__ double sh[8];
-    SumPair a;
-#pragma unroll 4
-    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += MSUM_BLOCKS * 256LL) a.add(mask[i]);
-    const double s = block_sum(a.value(), sh);
+    const double a = thread_sum(blockIdx.x * 256LL + threadIdx.x, n, MSUM_BLOCKS * 256, [&](long long i) { return mask[i]; });
+    const double s = block_sum(a, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
@@ -704,26 +722,22 @@ __device__ __forceinline__ double mask_sum(const double* part)
 
 // dY = 2 mask (Y - T) / sum(mask): FP32 (bp x nout), bf16 rows (bp x opad) and
 // bf16 transposed (nout x bp); per-block FP64 partial sums of the loss. The
-// factor 2 / sum and the squares are FP32 pairs (see SumPair); a block covers
-// LOSS_PT x 256 elements.
+// squares and the scaling are FP64 (an FP32 square leaves the range from an error
+// of 1.9e19 on); a block covers LOSS_PT x 256 elements.
 constexpr int LOSS_PT = 2;
 __global__ void __launch_bounds__(256) k_loss(const float* Y, const float* T, const float* mask, int batch, int nout,
                                               int opad, int bp, const double* mpart, float* dY, bf16* dYb, bf16* dYT,
                                               double* partial)
 {
     __shared__ double sh[8];
-    __shared__ float factor[2];
+    __shared__ double scale;  // 2 / sum
     if (threadIdx.x < 32) {
-        const double ms = mask_sum(mpart);
-        if (threadIdx.x == 0) {
-            const double q = 2.0 / ms;
-            factor[0] = (float)q;
-            factor[1] = (float)(q - (double)(float)q);
-        }
+        const double s = mask_sum(mpart);
+        if (threadIdx.x == 0) scale = 2.0 / s;
     }
     __syncthreads();
-    const float sc = factor[0], scl = factor[1];
-    SumPair l;
+    const double sc = scale;
+    double l = 0.0;
 #pragma unroll
     for (int k = 0; k < LOSS_PT; ++k) {
         const int i = (blockIdx.x * LOSS_PT + k) * 256 + threadIdx.x;
@@ -733,10 +747,9 @@ __global__ void __launch_bounds__(256) k_loss(const float* Y, const float* T, co
             if (r < batch) {
                 float m = mask[(size_t)r * nout + c];
                 float e = (Y[(size_t)r * nout + c] - T[(size_t)r * nout + c]) * m;
-                const float q = __fmul_rn(e, e);
-                l.add(q);
-                l.add(__fmaf_rn(e, e, -q));
-                d = __fmaf_rn(e, sc, __fmul_rn(e, scl));
+                const double ed = (double)e;
+                l = fma(ed, ed, l);
+                d = (float)(ed * sc);
             }
             dY[i] = d;
             bf16 b = __float2bfloat16_rn(d);
@@ -744,7 +757,7 @@ __global__ void __launch_bounds__(256) k_loss(const float* Y, const float* T, co
             dYT[(size_t)c * bp + r] = b;
         }
     }
-    const double sum = block_sum(l.value(), sh);
+    const double sum = block_sum(l, sh);
     if (threadIdx.x == 0) partial[blockIdx.x] = sum;
 }
 
@@ -760,7 +773,7 @@ __device__ __forceinline__ float adam_one(float p, float gi, float* m, float* v,
 
 // What follows the weight products, for a group of layers (blockIdx.y): the
 // weight gradients as the ordered sums of their parts, the bias gradients as
-// column sums of dZ (48 bits, fixed order), and with `adam` the update of the
+// column sums of dZ (FP64, fixed order), and with `adam` the update of the
 // parameters and their BF16 shadows (nothing is updated once *err is set).
 // Blocks [0, nw) hold 256 weights each, the next ones 8 bias columns each
 // (256 threads: 32 row strides of 8 columns), the last one (of layer group 0)
@@ -827,12 +840,7 @@ __global__ void __launch_bounds__(256) k_finish(const __grid_constant__ Finish f
     }
     const int c = (bx - f.nw) * 8 + (t & 7);
     if ((bx - f.nw) * 8 >= l.dout) return;
-    SumPair a;
-    if (c < l.dout) {
-#pragma unroll 8
-        for (int r = t >> 3; r < f.bp; r += 32) a.add(l.dZ[(size_t)r * l.dout + c]);
-    }
-    sh[t] = a.value();
+    sh[t] = c < l.dout ? thread_sum(t >> 3, f.bp, 32, [&](long long r) { return l.dZ[r * l.dout + c]; }) : 0.0;
     __syncthreads();
     for (int k = 128; k >= 8; k >>= 1) {
         if (t < k) sh[t] += sh[t + k];
