@@ -575,6 +575,34 @@ __global__ void __launch_bounds__(256) k_ball_direct(Params P, const float* dn,
 // ---------------------------------------------------------------------------
 constexpr int TAIL_WARPS = 8;
 
+// The sums of one node over the terms of the shell alone, in the kernel's order. The
+// kernel also multiplies the neighbours that its chunks of four dx reach outside the
+// shell, by zero coefficients; a node whose sums are not finite takes them from
+// here, so that an infinite density reaches only the nodes whose shell holds it.
+__device__ __noinline__ void tail_shell_only(const float* p, const TailRow* rows, int nrows, const float4* coef,
+                                             float t[3])
+{
+    for (int w = 0; w < TAIL_WARPS; ++w) {
+        float s[3] = {0.f, 0.f, 0.f};
+        for (int r = w; r < nrows; r += TAIL_WARPS) {
+            const TailRow row = rows[r];
+            float rs = 0.f, rd = 0.f;
+            for (int j = 0; j < 4 * row.count; ++j) {
+                const float* c = reinterpret_cast<const float*>(coef + row.coef + 2 * (j / 4)) + j % 4;
+                if (c[0] == 0.f && c[4] == 0.f) continue;
+                const int dx = 4 * row.first + j;
+                const float a = p[row.off + dx] - p[-row.off - dx], b = p[row.off - dx] - p[dx - row.off];
+                rs = fmaf(c[0], a + b, rs);
+                rd = fmaf(c[4], a - b, rd);
+            }
+            s[0] += rd;
+            s[1] = fmaf(row.dy, rs, s[1]);
+            s[2] = fmaf(row.dz, rs, s[2]);
+        }
+        for (int c = 0; c < 3; ++c) t[c] = w ? t[c] + s[c] : s[c];
+    }
+}
+
 __global__ void __launch_bounds__(32 * TAIL_WARPS, 2) k_tail(Params P, const float* __restrict__ dn,
                                                           const TailRow* __restrict__ rows, int nrows,
                                                           const float4* __restrict__ coef, float4* __restrict__ Ft)
@@ -661,6 +689,7 @@ __global__ void __launch_bounds__(32 * TAIL_WARPS, 2) k_tail(Params P, const flo
 #pragma unroll
         for (int w = 1; w < TAIL_WARPS; ++w) t[c] += part[w][3 * warp + c][lane];
     }
+    if (!isfinite(t[0] + t[1] + t[2])) tail_shell_only(base + warp, rows, nrows, coef, t);
     const float pre = P.sl[s].rho0 * (1.f + __ldg(base + warp));
     Ft[((long long)z * g.ny + y) * g.nx + x + warp] = make_float4(pre * t[0], pre * t[1], pre * t[2], 0.f);
 }
