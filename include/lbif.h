@@ -221,8 +221,8 @@ int lbif_batch_profiles(lbif_handle h, double* n_z, double* ux_z, int32_t hmax);
  * runs one pass: each node gathers the populations streaming into it (pull
  * form), applies the collision of their source node, and forms the moments
  * n, u of the next step from the values it holds, so the populations are
- * read and written once per step (tiles of 128 nodes marching in z; cross-
- * sections of at most 64 nodes run whole planes per CTA, with the same
+ * read and written once per step (tiles of 128 nodes marching in z; small
+ * cross-sections, of at most 128 nodes, run whole planes per CTA, with the same
  * arithmetic and identical results). Populations are stored as their non-equilibrium parts
  * relative to the equilibrium of their own node, which this pull form
  * decodes from the staged moments of the source node; the earlier two-pass

@@ -183,8 +183,8 @@ cudaError_t launch_tail_spectral(const Params& P, const float* dn, int D, float2
 // current plane is collided, 2 one plane per round, the gathers brought in by
 // the tensor-memory accelerator from pmap (a 4-D map of pin: x, y, z,
 // direction, box from pop_box; two-buffer layout only; bit 4 of status
-// records a bounded wait that ran out). Forms 1 and 2 need csm_ok grids; cross-
-// sections of at most 64 nodes run whole planes per CTA (lz, prefetch unused).
+// records a bounded wait that ran out). Forms 1 and 2 need csm_ok grids; small
+// cross-sections run whole planes per CTA in form 0 (lz unused).
 bool csm_ok(const Geom& g);
 cudaError_t launch_csm(const Params& P, const void* pin, void* pout, const CsmIO& io, const float4* F,
                        int* status, int lz, int prefetch, cudaStream_t s, const CUtensorMap* pmap = nullptr);

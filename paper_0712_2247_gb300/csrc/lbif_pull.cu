@@ -1120,17 +1120,23 @@ __global__ void __launch_bounds__(CSM_THREADS, 4)
 // forms and uses the quantities as in the marched forms (identical results).
 // 2048 slits of 4 x 4 x H: one node per thread without staging, each forming
 // its ~35 sources' quantities itself, 339 us; so 225 us.
+// Cross-sections of up to BLOCK_A_MAX nodes run so too where the marched tiles
+// would be less than two thirds full. Microseconds in tiles / whole planes: 65 x 1 x
+// 1600 28.9 / 17.4 (25.3 without staging), 33 x 2 x 1500 28.8 / 16.5, 13 x 6 x 20000
+// 133 / 124, 11 x 11 x 20000 216 / 180, but 25 x 4 x 20000 156 / 164 and
+// 16 x 8 x 20000 141 / 166.
 // (Writing the new moments through shared memory as whole padded planes, images
 // and all, instead of node by node: 217 us at 4 x 4, but 445 us against 372 at
 // 8 x 8; not kept.)
-constexpr int BLOCK_A = 64, BLOCK_NT = 256, BLOCK_NS = BLOCK_NT + 2 * BLOCK_A;
+constexpr int BLOCK_A = 64, BLOCK_A_MAX = 128, BLOCK_NT = 256;
 
-template <typename T, bool IP>
+template <typename T, bool IP, int AMAX>
 __global__ void __launch_bounds__(BLOCK_NT) k_pull_block(Params P, const T* pin, T* pout, CsmIO io,
                                                          const float4* F, int tz, int* status)
 {
     step_begin(P);
-    __shared__ float st[CSM_NF * BLOCK_NS];
+    constexpr int NS = BLOCK_NT + 2 * AMAX;  // staged nodes
+    __shared__ float st[CSM_NF * NS];
     constexpr bool RAW = F16_RAW<T>;
     const Geom& g = P.g;
     const int nx = g.nx, ny = g.ny, A = nx * ny, z0 = blockIdx.x * tz;
@@ -1156,7 +1162,7 @@ __global__ void __launch_bounds__(BLOCK_NT) k_pull_block(Params P, const T* pin,
         const int p = pidx(g, kx, ky, r);
         const float4 f = F[(long long)w * A + kxy];
         src_terms(ldp(io.dn + p), ldp(io.ux + p), ldp(io.uy + p), ldp(io.uz + p), f.x, f.y, f.z, f.w,
-                  P.sl[ks].inv_tau, shifted, [&](int j, float val) { st[j * BLOCK_NS + k] = val; });
+                  P.sl[ks].inv_tau, shifted, [&](int j, float val) { st[j * NS + k] = val; });
     }
     __syncthreads();
     if (!act) return;
@@ -1166,14 +1172,14 @@ __global__ void __launch_bounds__(BLOCK_NT) k_pull_block(Params P, const T* pin,
     }
     const int xo[3] = {x, x > 0 ? x - 1 : nx - 1, x < nx - 1 ? x + 1 : 0};  // sources with c_x = 0, 1, -1
     const int yo[3] = {y * nx, (y > 0 ? y - 1 : ny - 1) * nx, (y < ny - 1 ? y + 1 : 0) * nx};
-    using Src = Strided<BLOCK_NS>;
+    using Src = Strided<NS>;
     auto src = [&](auto ic) {
         constexpr int i = decltype(ic)::value;
         constexpr int cx = kCx(i), cy = kCy(i), cz = kCz(i);
         return Src{st + (zl + 1 - cz) * A + yo[cy > 0 ? 1 : (cy < 0 ? 2 : 0)] + xo[cx > 0 ? 1 : (cx < 0 ? 2 : 0)]};
     };
     const Src own{st + (zl + 1) * A + xy};
-    const float dnr = own.get<SQ_DN>();
+    const float dnr = own.template get<SQ_DN>();
     float d79, ux, uy, uz;
     pull_gather(src, own, (1.f - P.sl[s].inv_tau) / store_scale<T>(), dnr, bb, v, d79);
     const float dn =
@@ -1193,8 +1199,8 @@ static cudaError_t pull_block(const Params& P, const void* pin, void* pout, cons
     const int share = (g.nz + 2 * NUM_SMS - 1) / (2 * NUM_SMS);
     if (tz > share) tz = share;
     const int threads = (tz * A + 31) / 32 * 32;
-    return launch_step(k_pull_block<T, IP>, (g.nz + tz - 1) / tz, threads, 0, s, P, (const T*)pin, (T*)pout, io, F, tz,
-                       status);
+    const auto kernel = A <= BLOCK_A ? k_pull_block<T, IP, BLOCK_A> : k_pull_block<T, IP, BLOCK_A_MAX>;
+    return launch_step(kernel, (g.nz + tz - 1) / tz, threads, 0, s, P, (const T*)pin, (T*)pout, io, F, tz, status);
 }
 
 bool csm_ok(const Geom& g) { return g.nx >= CSM_TX && g.ny >= CSM_TY; }
@@ -1256,23 +1262,27 @@ static cudaError_t pull_pair(const Params& P, const void* pin, void* pout, const
     return launch_step(k_pull_pair<T, IP, TX>, (unsigned)blocks, CSM_THREADS, smem, s, P, pp, io, F, lz, tx, ty, status);
 }
 
-// The tile's width: the one that covers the cross-section with the least work,
+// The marched tiles' width: the one that covers the cross-section with the least work,
 // a tile of 16 or 8 columns counted 1.15 and 1.4 times one of 32 (its rows are
 // 64 or 32 bytes a warp load). With 32 / 16 / 8 columns: 203 x 117 x 75 112 / 121
 // / 154 us, a stack of 100 slits of 33 x 35 485 / 424 / 489 us, 7 x 300 x 100 50 /
 // 31 / 25 us, 100 slits of 48 x 24 (FP16 in place) 332 / 264 / 368 us.
-static int pair_width(const Geom& g)
+struct PairTiles {
+    int width;
+    long long nodes;  // that the tiles hold per plane
+};
+static PairTiles pair_tiles(const Geom& g)
 {
     const int w[] = {32, 16, 8};
     const double f[] = {1.0, 1.15, 1.4};
-    int best = 32;
+    PairTiles best{32, 0};
     double cost = 1e300;
     for (int k = 0; k < 3; ++k) {
         const int ty = CSM_THREADS / w[k];
-        const double c = f[k] * ((g.nx + w[k] - 1) / w[k]) * ((g.ny + ty - 1) / ty);
-        if (c < cost) {
-            cost = c;
-            best = w[k];
+        const long long n = (long long)((g.nx + w[k] - 1) / w[k]) * ((g.ny + ty - 1) / ty);
+        if (f[k] * n < cost) {
+            cost = f[k] * n;
+            best = PairTiles{w[k], n * CSM_THREADS};
         }
     }
     return best;
@@ -1282,8 +1292,11 @@ template <typename T, bool IP>
 static cudaError_t pull_any(const Params& P, const void* pin, void* pout, const CsmIO& io, const float4* F,
                             int* status, int lz, cudaStream_t s)
 {
-    if ((long long)P.g.nx * P.g.ny <= BLOCK_A) return pull_block<T, IP>(P, pin, pout, io, F, status, s);
-    switch (pair_width(P.g)) {
+    const long long A = (long long)P.g.nx * P.g.ny;
+    const PairTiles tiles = pair_tiles(P.g);
+    if (A <= BLOCK_A || (A <= BLOCK_A_MAX && 2 * tiles.nodes > 3 * A))
+        return pull_block<T, IP>(P, pin, pout, io, F, status, s);
+    switch (tiles.width) {
     case 32: return pull_pair<T, IP, 32>(P, pin, pout, io, F, status, lz, s);
     case 16: return pull_pair<T, IP, 16>(P, pin, pout, io, F, status, lz, s);
     default: return pull_pair<T, IP, 8>(P, pin, pout, io, F, status, lz, s);
