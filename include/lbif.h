@@ -249,7 +249,7 @@ int lbif_selftest_wait(int64_t polls, int32_t* timed_out);
  * current state (trials launches each) and keep the fastest: the ball
  * kernel's CTA target and its plane staging (1 = tensor-memory-accelerator
  * copies, 0 = plain loads), the force kernel's tile-group edge, and the pull
- * pass's z planes per CTA segment (8, 16, 32) and its gathers (plain; the
+ * pass's z planes per CTA segment (the library's choice, 8, 16, 32) and its gathers (plain; the
  * next plane's populations loaded while the current one is collided; or the
  * per-direction source boxes of each tile copied into shared memory one plane
  * ahead by the tensor-memory accelerator, two-buffer handles whose x rows

@@ -1382,7 +1382,7 @@ extern "C" int lbif_autotune(lbif_handle h, int32_t trials, int32_t* ball_want, 
             best_group = gsz;
         }
     }
-    // Pull pass: z planes per CTA segment x gathers (plain, prefetched one
+    // Pull pass: z planes per CTA segment x gathers (two planes at a time, prefetched one
     // plane ahead, tensor-memory-accelerator boxes when the handle has
     // population maps). A trial reads the
     // current populations and fields and writes only the next step's buffers
@@ -1396,10 +1396,13 @@ extern "C" int lbif_autotune(lbif_handle h, int32_t trials, int32_t* ball_want, 
         float* const* u = h->u[h->fcur];
         float* const* w = h->u[h->fcur ^ 1];
         CsmIO io{h->dn[h->fcur], u[0], u[1], u[2], h->dn[h->fcur ^ 1], w[0], w[1], w[2]};
-        const int lzs[] = {8, 16, 32};
+        // 0, the length chosen from the grid (2 .. 32 planes), first: it stays unless
+        // another one is faster. The one-plane forms take 16 for it.
+        const int lzs[] = {0, 8, 16, 32};
         best = 1e30f;
         for (int pf = 0; pf <= (h->pop_map_ok ? 2 : 1); ++pf)
             for (int lz : lzs) {
+                if (pf && !lz) continue;
                 float tot = 0.f;
                 for (int k = 0; k < trials + 1; ++k) {
                     CK(h, cudaEventRecord(e0, h->stream));
