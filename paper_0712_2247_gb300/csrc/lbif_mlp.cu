@@ -1043,6 +1043,13 @@ extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32
         mlp_free(m);
         return mfail(nullptr, LBIF_ERR_CUDA, "lbif_mlp_create: shared memory configuration failed");
     }
+    // the zero fills above went to the default stream, which a non-blocking stream of
+    // the caller's does not wait for: they end before the first call can write
+    if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+        cudaGetLastError();
+        mlp_free(m);
+        return mfail(nullptr, LBIF_ERR_CUDA, "lbif_mlp_create: zero fill failed");
+    }
     *out = m;
     return LBIF_OK;
 }
