@@ -26,10 +26,6 @@ __device__ __forceinline__ constexpr int kCz(int i)
     return (i == 5 || i == 11 || i == 14 || i == 15 || i == 18) ? 1
          : (i == 6 || i == 12 || i == 13 || i == 16 || i == 17) ? -1 : 0;
 }
-__device__ __forceinline__ constexpr float kW(int i)
-{
-    return i == 0 ? 1.f / 3.f : (i <= 6 ? 1.f / 18.f : 1.f / 36.f);
-}
 // |c_i|^2 (0, 1 or 2 on D3Q19)
 __device__ __forceinline__ constexpr int kC2(int i) { return kCx(i) * kCx(i) + kCy(i) * kCy(i) + kCz(i) * kCz(i); }
 __device__ __forceinline__ constexpr int opp_of(int i) { return i == 0 ? 0 : ((i & 1) ? i + 1 : i - 1); }
@@ -54,7 +50,10 @@ __device__ __forceinline__ float ldq(const __half* p)
     else
         return ldp(p);
 }
-__device__ __forceinline__ float late_cvt(float bits) { return __half2float(__ushort_as_half((unsigned short)__float_as_int(bits))); }
+__device__ __forceinline__ float late_cvt(float bits)
+{
+    return __half2float(__ushort_as_half((unsigned short)__float_as_int(bits)));
+}
 __device__ __forceinline__ void stp(float* p, float v) { *p = v; }
 __device__ __forceinline__ void stp(__half* p, float v) { *p = __float2half_rn(v); }
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
@@ -168,34 +167,6 @@ __device__ __forceinline__ bool flat_node(const Geom& g, const TileMap& tm, int 
 // slit of plane z (-1 for a gap plane between stacked slits)
 __device__ __forceinline__ int slit_of(const Params& P, int z) { return __ldg(P.zslit + z); }
 __device__ __forceinline__ bool frozen(const Params& P, int s) { return __ldg(P.done + s) != 0; }
-
-// acc += c x for a lattice-velocity component c in {-1, 0, 1} known after
-// unrolling (a product with a zero component is not folded under IEEE rules,
-// so the zero case must not be written as one)
-__device__ __forceinline__ void add_c(float& acc, int c, float x)
-{
-    if (c > 0) acc += x;
-    if (c < 0) acc -= x;
-}
-
-// c_i . (x, y, z), adding only the nonzero components (in increasing axis
-// order, as the full dot product rounds them)
-__device__ __forceinline__ float dot_c(int i, float x, float y, float z)
-{
-    const int cx = kCx(i), cy = kCy(i), cz = kCz(i);
-    if (cx != 0) {
-        float r = cx > 0 ? x : -x;
-        add_c(r, cy, y);
-        add_c(r, cz, z);
-        return r;
-    }
-    if (cy != 0) {
-        float r = cy > 0 ? y : -y;
-        add_c(r, cz, z);
-        return r;
-    }
-    return cz > 0 ? z : (cz < 0 ? -z : 0.f);
-}
 
 __host__ __device__ constexpr int cisqrt(int n)
 {

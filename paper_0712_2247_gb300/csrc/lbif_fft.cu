@@ -494,9 +494,11 @@ void fft_lines(float2* data, int L, int nx, long long nlines, bool along_y, cons
     if (along_y)
         k_fft<GL, true><<<blocks, FFT_THREADS, smem, s>>>(data, L, ilog2(L), ilog2(nx), nlines, tw, inverse, e);
     else if (ends_mode == 1)
-        k_fft<GL, false, true, false><<<blocks, FFT_THREADS, smem, s>>>(data, L, ilog2(L), ilog2(nx), nlines, tw, inverse, e);
+        k_fft<GL, false, true, false><<<blocks, FFT_THREADS, smem, s>>>(data, L, ilog2(L), ilog2(nx), nlines, tw, inverse,
+                                                                         e);
     else if (ends_mode == 2)
-        k_fft<GL, false, false, true><<<blocks, FFT_THREADS, smem, s>>>(data, L, ilog2(L), ilog2(nx), nlines, tw, inverse, e);
+        k_fft<GL, false, false, true><<<blocks, FFT_THREADS, smem, s>>>(data, L, ilog2(L), ilog2(nx), nlines, tw, inverse,
+                                                                         e);
     else
         k_fft<GL, false><<<blocks, FFT_THREADS, smem, s>>>(data, L, ilog2(L), ilog2(nx), nlines, tw, inverse, e);
 }
@@ -539,7 +541,8 @@ bool tail_spectral_ok(const Geom& g)
 size_t tail_spectral_bytes(const Geom& g, int D)
 {
     const size_t nxy = (size_t)g.nx * g.ny;
-    return sizeof(float4) * (D + 1) * nxy + sizeof(float2) * (3 * nxy * (size_t)g.nz + g.nx / 2 + g.ny / 2 + (g.nz + 1) / 2);
+    return sizeof(float4) * (D + 1) * nxy +
+           sizeof(float2) * (3 * nxy * (size_t)g.nz + g.nx / 2 + g.ny / 2 + (g.nz + 1) / 2);
 }
 
 // Layout of the work buffer: Kb ((D+1) x ny x nx float4), Pp and O2 (together)

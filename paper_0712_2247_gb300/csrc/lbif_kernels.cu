@@ -1002,7 +1002,6 @@ cudaError_t launch_ball(const Params& P, const float* dn, float* dG, int* status
         case 4: return launch_step(k_ball_direct<4>, nb, nt, 0, s, P, dn, dG, status, skip_done);
         default: return launch_step(k_ball_direct<0>, nb, nt, 0, s, P, dn, dG, status, skip_done);
         }
-        return cudaGetLastError();
     }
     switch (P.sigma / 2) {
     case 1: return ball_r<1>(P, dn, dG, status, want, skip_done, tmap, s);

@@ -594,7 +594,8 @@ __global__ void __launch_bounds__(256, 2) k_mlp_forward(const __grid_constant__ 
                         if (c + 16 <= f.nout && ((uintptr_t)y & 15) == 0) {
 #pragma unroll
                             for (int q = 0; q < 4; ++q)
-                                reinterpret_cast<float4*>(y)[q] = make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
+                                reinterpret_cast<float4*>(y)[q] =
+                                    make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
                         } else {
 #pragma unroll
                             for (int j = 0; j < 16; ++j)
@@ -703,7 +704,8 @@ constexpr int MSUM_BLOCKS = 64;
 __global__ void __launch_bounds__(256) k_msum(const float* mask, long long n, double* part)
 {
     __shared__ double sh[8];
-    const double a = thread_sum(blockIdx.x * 256LL + threadIdx.x, n, MSUM_BLOCKS * 256, [&](long long i) { return mask[i]; });
+    const double a =
+        thread_sum(blockIdx.x * 256LL + threadIdx.x, n, MSUM_BLOCKS * 256, [&](long long i) { return mask[i]; });
     const double s = block_sum(a, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
@@ -886,7 +888,6 @@ struct lbif_mlp_ctx {
     std::vector<size_t> wpoff;   // offsets of the layers in it
     std::vector<float*> Z;       // pre-activations per layer (bp x dout)
     std::vector<bf16*> H, HT;    // layer inputs (bp x kpad) and transposed (kpad x bp)
-    float* dY = nullptr;         // output error FP32 (bp x nout)
     std::vector<float*> dZ;      // per layer FP32 error (bp x dout)
     std::vector<bf16*> dZb, dZT; // bf16 copies
     float* dWpart = nullptr;     // parts of the weight products: splits x npart
@@ -937,7 +938,8 @@ static int mfail(lbif_mlp_ctx* m, int code, const std::string& s)
 static void mlp_free(lbif_mlp_ctx* m)
 {
     if (!m) return;
-    std::vector<void*> bufs = {m->Wp, m->p, m->g, m->m, m->v, m->dY, m->dWpart, m->Xd, m->Td, m->Md, m->Yd, m->partial, m->mpart, m->err};
+    std::vector<void*> bufs = {m->Wp, m->p, m->g, m->m, m->v, m->dWpart, m->Xd, m->Td, m->Md,
+                               m->Yd, m->partial, m->mpart, m->err};
     for (auto* b : m->Wb) bufs.push_back(b);
     for (auto* b : m->WTb) bufs.push_back(b);
     for (auto* b : m->Z) bufs.push_back(b);
@@ -965,7 +967,10 @@ static bool dalloc(T** p, size_t n)
 
 // shared memory of the fused forward: activations of 128 rows x kmax, the ring
 // of weight chunks, barriers and the TMEM address slot
-static int fused_smem(int kmax, int nmax) { return 256 * kmax + FUSE_RING * nmax * FUSE_KC * 2 + 8 * (2 * FUSE_RING + 1) + 16; }
+static int fused_smem(int kmax, int nmax)
+{
+    return 256 * kmax + FUSE_RING * nmax * FUSE_KC * 2 + 8 * (2 * FUSE_RING + 1) + 16;
+}
 
 extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32_t nhidden, int32_t nout,
                                int32_t max_batch, void* stream)
@@ -1007,7 +1012,7 @@ extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32
     }
     const int bp = m->bp_max;
     bool ok = dalloc(&m->p, off) && dalloc(&m->g, off) && dalloc(&m->m, off) && dalloc(&m->v, off) &&
-              dalloc(&m->dY, (size_t)bp * nout) && dalloc(&m->dWpart, wgrad_splits(bp) * m->npart) &&
+              dalloc(&m->dWpart, wgrad_splits(bp) * m->npart) &&
               dalloc(&m->Xd, (size_t)max_batch * nin) && dalloc(&m->Td, (size_t)max_batch * nout) &&
               dalloc(&m->Md, (size_t)max_batch * nout) && dalloc(&m->Yd, (size_t)bp * nout) &&
               dalloc(&m->partial, (size_t)(bp * nout + 255) / 256 + 1) && dalloc(&m->mpart, MSUM_BLOCKS) &&
@@ -1038,7 +1043,8 @@ extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32
     }
     if (cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256)) != cudaSuccess ||
         cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256)) != cudaSuccess ||
-        cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, fused_smem(256, 256)) != cudaSuccess) {
+        cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, fused_smem(256, 256)) !=
+            cudaSuccess) {
         cudaGetLastError();
         mlp_free(m);
         return mfail(nullptr, LBIF_ERR_CUDA, "lbif_mlp_create: shared memory configuration failed");
@@ -1203,7 +1209,8 @@ static int pack_input(lbif_mlp_ctx* m, const float* X, int batch, int on_device)
 static int check_err(lbif_mlp_ctx* m)
 {
     MCK(m, cudaStreamSynchronize(m->stream));
-    if (*(volatile double*)(m->host + 1) != 0.0) return mfail(m, LBIF_ERR_TIMEOUT, "tensor-core product did not complete within its wait limit");
+    if (*(volatile double*)(m->host + 1) != 0.0)
+        return mfail(m, LBIF_ERR_TIMEOUT, "tensor-core product did not complete within its wait limit");
     return LBIF_OK;
 }
 

@@ -663,7 +663,10 @@ constexpr int PAIR_MINB = 4;  // CTAs per SM
 
 __host__ __device__ constexpr int ab_of(int k)
 {
-    return k == SQ_DN ? AB_DN : (k < SQ_CA ? AB_P + (k - SQ_P) : (k == SQ_CA + 2 ? AB_CZ : (k < SQ_X ? AB_CP + (k - SQ_CP - 1) : AB_X + (k - SQ_X - 1))));
+    return k == SQ_DN ? AB_DN
+         : k < SQ_CA ? AB_P + (k - SQ_P)
+         : k == SQ_CA + 2 ? AB_CZ
+         : k < SQ_X ? AB_CP + (k - SQ_CP - 1) : AB_X + (k - SQ_X - 1);
 }
 __host__ __device__ constexpr bool in_ow(int k) { return k == SQ_CA || k == SQ_CA + 1 || k == SQ_CP || k == SQ_X; }
 __host__ __device__ constexpr int ow_of(int k) { return k == SQ_CP ? OW_CP : (k == SQ_X ? OW_X : OW_C + (k - SQ_CA)); }
