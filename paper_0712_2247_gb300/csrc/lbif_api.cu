@@ -441,6 +441,7 @@ static int create_impl(lbif_handle* out, int nx, int ny, int nz, int sigma, int 
     }
     const double kT = 1.0 / 3.0;
     P.sigma = sigma;
+    P.ball_z = ball_chunk(g, sigma);
     P.kappa = (float)(2.0 / (sqrt(kT) * sqrt(M_PI)));
     P.inv_sigma = (float)(1.0 / sigma);
     P.ball_inv = (float)(1.0 / ball_count(sigma));
@@ -1334,7 +1335,7 @@ extern "C" int lbif_autotune(lbif_handle h, int32_t trials, int32_t* ball_want, 
     cudaEvent_t e0, e1;
     CK(h, cudaEventCreate(&e0));
     CK(h, cudaEventCreate(&e1));
-    const int balls[] = {304, 608, 1216, 2432, 4864};
+    const int balls[] = {ball_ctas(P), 304, 608, 1216, 2432, 4864};  // the default's number first
     const int groups[] = {64, 128, 256, 1 << 20};
     float best = 1e30f;
     int best_ball = 0, best_group = 0;

@@ -83,6 +83,7 @@ struct Params {
     float inv_sigma;
     float ball_inv;  // 1 / ball node count
     int sigma;
+    int ball_z;      // z planes per CTA of the ball kernel (ball_chunk)
     int hs, coupling, regularize, g2form, tail, storage;
     int c2;               // energy source of Eq. C2eq on (F.w carries C2 / n0)
     int shifted;          // velocity-shifted second-order forcing (equilibrium at u + F/(2n))
@@ -140,7 +141,10 @@ cudaError_t launch_pop_canon(const Params& P, void* pop, int i, void* canon, int
 // the four fields <-> four unpadded N-arrays (checkpoints)
 cudaError_t launch_write_fields(const Params& P, const float* src, float* const f[4], cudaStream_t s);
 cudaError_t launch_read_fields(const Params& P, const float* const f[4], float* out, cudaStream_t s);
-// want: CTAs to aim for when splitting z into chunks (<= 0: default).
+// z planes per CTA of the ball kernel on this grid, and the CTAs that makes
+int ball_chunk(const Geom& g, int sigma);
+int ball_ctas(const Params& P);
+// want: CTAs to aim for when splitting z into chunks (<= 0: chunks of P.ball_z planes).
 // tmap: a 3-D tensor map of dn (padded extents px, py, pz; box from
 // ball_box) to stage the plane tiles with the tensor-memory accelerator, or
 // NULL for plain loads. Bit 4 of status records a bounded wait that ran out.

@@ -6,6 +6,8 @@
 // (dn = n/n0 - 1, dG = g2 - g2(eta0)), and mirror-image quadrature points are
 // combined before they are summed, so a uniform state gives an exactly zero
 // force. FP64 appears only in the profile / mass reductions.
+#include <math.h>
+
 #include <atomic>
 #include <utility>
 
@@ -930,6 +932,47 @@ cudaError_t launch_read_fields(const Params& P, const float* const f[4], float* 
     return cudaGetLastError();
 }
 
+// z planes per CTA of the ball kernel: more CTAs fill the SMs, but each reads 2 R
+// planes beyond its own. The length is the one that minimises
+//   (planes + 2 R + 5) (1 + b k),  k = CTAs per SM,  b = 0.05 + 0.015 R^1.5,
+// 5 standing for a CTA's start and b for what a co-resident CTA adds to the time of a
+// plane (it grows with the radius as the row and disc sums take over from the
+// latencies); up to five, CTAs per SM count whole. Over 26 grids (R 1 to 12, 2 to
+// 512 tiles, 8 to 11,000 planes, every length timed) it lies within 9 % of the best
+// length, 2 % on average. Microseconds with 1216 CTAs of at least 2 R planes (R or R / 2
+// where those are few) / so: 203 x 117 x 75, sigma 10 55.6 / 45.6, sigma 24 196 / 151,
+// 400 x 300 x 20, sigma 12 73.4 / 65.2, 128^3, sigma 18 107 / 94, 64 x 64 x 128, sigma 8
+// 20.6 / 20.5, 256 x 256 x 128, sigma 8 90.4 / 92.1, 512 x 512 x 192, sigma 12 531 / 537.
+int ball_chunk(const Geom& g, int sigma)
+{
+    const int R = sigma / 2;
+    const double b = 0.05 + 0.015 * R * sqrt((double)R);
+    const long long tiles = (long long)((g.nx + BALL_TX - 1) / BALL_TX) * ((g.ny + BALL_TY - 1) / BALL_TY);
+    int best = g.nz;
+    double cost = 1e300;
+    // up to 16 CTAs per SM, at most 48 numbers of chunks
+    long long most = 16LL * NUM_SMS / tiles;
+    if (most > g.nz) most = g.nz;
+    if (most < 1) most = 1;
+    const long long tries = most < 48 ? most : 48;
+    for (long long i = 1; i <= tries; ++i) {
+        const int chunks = (int)(most * i / tries), z = (g.nz + chunks - 1) / chunks;
+        const double q = (double)(tiles * ((g.nz + z - 1) / z)) / NUM_SMS;
+        const double c = (z + 2 * R + 5) * (1.0 + b * (q <= 5.0 ? ceil(q) : q));
+        if (c < cost) {
+            cost = c;
+            best = z;
+        }
+    }
+    return best;
+}
+
+int ball_ctas(const Params& P)
+{
+    const Geom& g = P.g;
+    return (g.nx + BALL_TX - 1) / BALL_TX * ((g.ny + BALL_TY - 1) / BALL_TY) * ((g.nz + P.ball_z - 1) / P.ball_z);
+}
+
 template <int R>
 static cudaError_t ball_r(const Params& P, const float* dn, float* dG, int* status, int want,
                          int skip_done, const CUtensorMap* tmap, cudaStream_t s)
@@ -953,24 +996,15 @@ static cudaError_t ball_r(const Params& P, const float* dn, float* dG, int* stat
         flags.fetch_or(bit);
     }
     int gx = (g.nx + BALL_TX - 1) / BALL_TX, gy = (g.ny + BALL_TY - 1) / BALL_TY;
-    // CTAs to aim for: about eight per SM (512 x 512 x 192, sigma 12: 608 / 1216 /
-    // 2432 / 4864 CTAs 0.606 / 0.554 / 0.564 / 0.625 ms in the former form; 256 x
-    // 256 x 128, sigma 8: 100 / 95 / 103 / 103 us). A chunk of z planes reads 2 R
-    // more, so chunks hold at least 2 R planes, unless that leaves fewer than three
-    // CTAs per SM (then R: 64 x 64 x 128, sigma 8, 24 -> 20 us; 256 x 256 x 64,
-    // sigma 10, with enough of them would lose 73 -> 80) or that fewer than one
-    // (then R / 2: 32 x 32 x 64, sigma 8, 23 / 16 / 14 us).
-    if (want <= 0) want = 8 * NUM_SMS;
-    int nchunk = (want + gx * gy - 1) / (gx * gy);
-    const long long tiles = (long long)gx * gy;
-    int least = 2 * R;
-    if (tiles * (g.nz / least) < 3 * NUM_SMS) least = R;
-    if (tiles * (g.nz / least) < NUM_SMS) least = (R + 1) / 2;
-    const int maxchunk = g.nz / least > 1 ? g.nz / least : 1;
-    if (nchunk > maxchunk) nchunk = maxchunk;
-    if (nchunk < 1) nchunk = 1;
-    int zchunk = (g.nz + nchunk - 1) / nchunk;
-    nchunk = (g.nz + zchunk - 1) / zchunk;
+    int zchunk = P.ball_z;
+    if (want > 0) {
+        // asked for: that many CTAs, of at least 2 R planes each (or the default's number)
+        const long long tiles = (long long)gx * gy;
+        const long long most = max(g.nz / (2 * R), (g.nz + zchunk - 1) / zchunk);
+        const long long n = min((want + tiles - 1) / tiles, most);
+        zchunk = (int)((g.nz + n - 1) / n);
+    }
+    const int nchunk = (g.nz + zchunk - 1) / zchunk;
     dim3 grid(gx, gy, nchunk);
     if (tmap)
         return launch_step(k_ball_tma<R>, grid, BALL_THREADS, smem, s, P, *tmap, dG, status, zchunk, skip_done);
