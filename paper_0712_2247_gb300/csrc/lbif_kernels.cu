@@ -1026,8 +1026,10 @@ cudaError_t launch_ball(const Params& P, const float* dn, float* dG, int* status
     // tile row (20 x 200 x 150, sigma 4: tiles 18, direct 14 us; 128 slits of 32 x 32:
     // tiles 58, direct 72 us)
     if (P.g.nx < (P.sigma <= 4 ? BALL_TX : BALL_TX / 2) || P.g.ny < BALL_TY / 2) {
-        // small blocks on small grids, so that the SMs share them
-        const int nt = P.g.N < 256LL * NUM_SMS ? 64 : 256;
+        // small blocks on small grids, so that the SMs share them; not for the loop over
+        // large radii, whose blocks share their many rows in L1 (2 x 75 x 29, sigma 24: 64
+        // threads 401 us, 256 threads 341; 3 x 70 x 12, sigma 12: 70 and 59)
+        const int nt = P.g.N < 256LL * NUM_SMS && P.sigma <= 8 ? 64 : 256;
         const unsigned nb = nblocks(P.g.N, nt);
         switch (P.sigma / 2) {
         case 1: return launch_step(k_ball_direct<1>, nb, nt, 0, s, P, dn, dG, status, skip_done);
