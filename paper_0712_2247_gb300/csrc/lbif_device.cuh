@@ -275,18 +275,10 @@ __device__ __forceinline__ IpSlots ip_slots(const Params& P, const SlitParam& S,
 // lets the successor come up. What it reads of its predecessors goes through
 // ordinary loads (ldp).
 //
-// The attribute is given up to 512 nodes per SM. Microseconds per step without /
-// with it at sigma 4 and 10: 8 x 8 x 16 20.8 / 16.5 and 50.5 / 48.1, 16 x 16 x 32
-// 26.4 / 20.3 and 41.3 / 35.2, 24 x 24 x 48 28.1 / 22.5 and 39.5 / 34.9,
-// 32 x 32 x 64 29.0 / 26.6 and 39.3 / 36.5, but 40 x 40 x 64 34.9 / 34.9 and
-// 43.6 / 53.0, 64^3 at sigma 4 43.2 / 44.4 and 512 x 512 x 192 4583 / 4713: there
-// the successor's blocks take places on the SMs, and wait in them, while the
-// predecessor still needs them.
-constexpr long long PDL_NODES = 512LL * NUM_SMS;
-
+// P.overlap says whether the attribute is given (step_overlap).
 __device__ __forceinline__ void step_begin(const Params& P)
 {
-    if (P.g.N > PDL_NODES) return;
+    if (!P.overlap) return;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
@@ -304,7 +296,7 @@ static inline cudaError_t launch_step(void (*kernel)(Params, K...), dim3 grid, d
     c.dynamicSmemBytes = smem;
     c.stream = s;
     c.attrs = &at;
-    c.numAttrs = P.g.N <= PDL_NODES ? 1 : 0;
+    c.numAttrs = P.overlap ? 1 : 0;
     return cudaLaunchKernelEx(&c, kernel, P, static_cast<K>(args)...);
 }
 

@@ -91,6 +91,7 @@ struct Params {
     const SlitParam* sl;  // device table, nslits entries
     const int* zslit;     // device table, nz entries
     const int* done;      // device flags, nslits entries (1 = frozen)
+    int overlap;          // the step's kernels overlap their launches (step_overlap)
     int inplace;          // populations in one buffer (shifting slots)
     const int4* clk;      // in place: per slit (t mod nx, t mod ny, t mod R) of its step t
     long long soff[Q];    // node-index offsets of the 19 neighbours (no wrap)
