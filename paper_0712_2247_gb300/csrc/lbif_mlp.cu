@@ -413,11 +413,14 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_wgrad(const __grid_constant
 // per element against 512 FLOP on the tensor core, so two CTAs share an SM and
 // one's epilogue covers the other's products. Four launches that passed the
 // activations through L2 took 234 us for 65,536 rows at 4 -> 3 x 256 -> 160; this
-// takes 134 us, 115 of them in the kernel (43 us of issue; an SM holds three or
+// takes 131 us, 115 of them in the kernel (43 us of issue; an SM holds three or
 // four of the 512 tiles). Loading the next chunk of accumulators and biases
-// early changed nothing.
+// early changed nothing. Up to one tile per SM a CTA runs 16 warps (NT 512), so that
+// the epilogue of an SM's only tile is shared by as many as two tiles': 1024 rows,
+// 256 -> 8 x 256 -> 256 139 -> 125 us together with the 16-byte input loads (126 as nine
+// launches), 4 -> 20 x 256 -> 160 260 -> 250 us (245).
 // ---------------------------------------------------------------------------
-constexpr int FUSE_KC = 32, FUSE_RING = 3;
+constexpr int FUSE_KC = 32, FUSE_RING = 3, FUSE_SMS = 152;  // SMs of a GB300
 
 // element (r, c) of a layer's weights in its packed image: chunks of FUSE_KC
 // columns (the last one shorter), each n16 rows of 8-row x 16-byte core
@@ -458,7 +461,8 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                  : "memory");
 }
 
-__global__ void __launch_bounds__(256, 2) k_mlp_forward(const __grid_constant__ Fused f)
+template <int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) k_mlp_forward(const __grid_constant__ Fused f)
 {
     extern __shared__ __align__(1024) uint8_t fsm[];
     uint8_t* const act = fsm;
@@ -514,15 +518,29 @@ __global__ void __launch_bounds__(256, 2) k_mlp_forward(const __grid_constant__ 
         // the input rows as BF16 core matrices, zero beyond nin and the batch
         {
             const int r = tid & 127, row = tile * 128 + r, kcore = kp0 / 8;
-            for (int kp = tid >> 7; kp < kcore; kp += 2) {
+            const float* x = f.X + (size_t)row * f.nin;
+            // 16-byte loads where every row starts on one (a warp's rows are apart, so
+            // a load costs the same whatever its width)
+            const bool wide = f.nin % 4 == 0 && ((uintptr_t)f.X & 15) == 0;
+            for (int kp = tid >> 7; kp < kcore; kp += NT / 128) {
+                float v[8];
+                if (wide) {
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int c = kp * 8 + 4 * e;
+                        const float4 a = row < f.batch && c < f.nin ? *reinterpret_cast<const float4*>(x + c)
+                                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+                        v[4 * e] = a.x, v[4 * e + 1] = a.y, v[4 * e + 2] = a.z, v[4 * e + 3] = a.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v[e] = row < f.batch && kp * 8 + e < f.nin ? x[kp * 8 + e] : 0.f;
+                }
                 uint4 pk;
                 uint32_t* w = reinterpret_cast<uint32_t*>(&pk);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const int c = kp * 8 + 2 * e;
-                    const float a = row < f.batch && c < f.nin ? f.X[(size_t)row * f.nin + c] : 0.f;
-                    const float b = row < f.batch && c + 1 < f.nin ? f.X[(size_t)row * f.nin + c + 1] : 0.f;
-                    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
                     w[e] = *reinterpret_cast<const uint32_t*>(&h);
                 }
                 *reinterpret_cast<uint4*>(act + ((r >> 3) * kcore + kp) * 128 + (r & 7) * 16) = pk;
@@ -567,7 +585,7 @@ __global__ void __launch_bounds__(256, 2) k_mlp_forward(const __grid_constant__ 
             if (!ok) break;
             const int lg = warp % 4, r = 32 * lg + lane, row = tile * 128 + r;
             if (tile * 128 + 32 * lg < f.batch) {  // the warp holds a row of the batch
-                for (int c = 16 * (warp / 4); c < N; c += 32) {
+                for (int c = 16 * (warp / 4); c < N; c += NT / 8) {
                     float v[16], z[16];
                     __syncwarp();  // rows past the batch skip the stores below
                     tmem_ld16(tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)c, v);
@@ -1043,7 +1061,9 @@ extern "C" int lbif_mlp_create(lbif_mlp* out, int32_t nin, int32_t hidden, int32
     }
     if (cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256)) != cudaSuccess ||
         cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(256)) != cudaSuccess ||
-        cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, fused_smem(256, 256)) !=
+        cudaFuncSetAttribute(k_mlp_forward<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, fused_smem(256, 256)) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(k_mlp_forward<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, fused_smem(256, 256)) !=
             cudaSuccess) {
         cudaGetLastError();
         mlp_free(m);
@@ -1186,8 +1206,11 @@ static int infer(lbif_mlp_ctx* m, const float* X, int batch, float* Y)
     // two CTAs per SM: shared memory keeps a third one (and its TMEM) out
     int smem = fused_smem(kmax, nmax);
     if (smem < 80 * 1024) smem = 80 * 1024;
-    const int grid = f.tiles < 304 ? f.tiles : 304;
-    k_mlp_forward<<<grid, 256, smem, m->stream>>>(f);
+    // up to one tile per SM: 16 warps a CTA, which share the epilogue of the only tile
+    if (f.tiles <= FUSE_SMS)
+        k_mlp_forward<512><<<f.tiles, 512, smem, m->stream>>>(f);
+    else
+        k_mlp_forward<256><<<f.tiles < 2 * FUSE_SMS ? f.tiles : 2 * FUSE_SMS, 256, smem, m->stream>>>(f);
     MCK(m, cudaGetLastError());
     return LBIF_OK;
 }
