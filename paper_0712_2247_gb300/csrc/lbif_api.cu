@@ -39,8 +39,10 @@ struct lbif_ctx {
     float4* Ft = nullptr;
     float4* F = nullptr;              // F / n0 per node (force kernel -> collision kernel)
     TailRow* tail_rows = nullptr;     // direct tail sum (no spectral path): its rows and coefficients
-    float4* tail_coef = nullptr;
+    float4* tail_coef = nullptr;      // (or, pair by pair, the weights of tail_off)
     int tail_nrows = 0;
+    int* tail_off = nullptr;          // padded offsets of the pairs, NULL when summed by rows
+    int tail_npairs = 0;
     float2* tail_work = nullptr;      // spectral tail: fields, kernel transform, twiddles
     int tail_D = 0;                   // z reach of the tail kernel (planes)
     bool tail_fft = false;
@@ -164,6 +166,7 @@ static const CUtensorMap* ball_map(const lbif_ctx* h, int i)
 static cudaError_t run_tail(lbif_ctx* h, const float* dn)
 {
     if (h->tail_fft) return launch_tail_spectral(h->P, dn, h->tail_D, h->tail_work, h->Ft, h->stream);
+    if (h->tail_off) return launch_tail_pairs(h->P, dn, h->tail_off, h->tail_coef, h->tail_npairs, h->Ft, h->stream);
     return launch_tail(h->P, dn, h->tail_rows, h->tail_nrows, h->tail_coef, h->Ft, h->stream);
 }
 
@@ -199,7 +202,7 @@ static void free_ctx(lbif_ctx* h)
 {
     if (!h) return;
     if (h->graph) cudaGraphExecDestroy(h->graph);
-    void* bufs[] = {h->pop[0], h->pop[1], h->Ft, h->F, h->tail_rows, h->tail_coef, h->tail_work, h->status_d,
+    void* bufs[] = {h->pop[0], h->pop[1], h->Ft, h->F, h->tail_rows, h->tail_coef, h->tail_off, h->tail_work, h->status_d,
                     h->prof_d, h->scratch, h->d_sl, h->d_zslit, h->d_done, h->clk_d};
     for (void* b : bufs)
         if (b) cudaFree(b);
@@ -308,12 +311,13 @@ static void tail_pairs(int sigma, double rcut, double eps, std::vector<int>& dxs
             }
 }
 
-// the same displacements as rows for the direct sum (see TailRow)
-static void tail_direct_rows(const Geom& g, int sigma, double rcut, double eps, std::vector<TailRow>& rows,
+// the same displacements as rows for the direct sum (see TailRow); returns their number
+static int tail_direct_rows(const Geom& g, int sigma, double rcut, double eps, std::vector<TailRow>& rows,
                              std::vector<float4>& coef)
 {
     const double rmax = rcut * sigma;
     const int R = (int)ceil(rmax);
+    int pairs = 0;
     for (int dz = 0; dz <= R; ++dz)
         for (int dy = (dz == 0 ? 0 : -R); dy <= R; ++dy) {
             std::vector<double> c(4 * (R / 4 + 1), 0.0);
@@ -322,7 +326,9 @@ static void tail_direct_rows(const Geom& g, int sigma, double rcut, double eps, 
                 const double r2 = (double)dx * dx + (double)dy * dy + (double)dz * dz;
                 if (r2 < (double)sigma * sigma || r2 > rmax * rmax) continue;
                 c[dx] = tail_slope(sigma, eps, r2);
-                if (dx == 0 || (dy == 0 && dz == 0)) c[dx] *= 0.5;
+                const bool half = dx == 0 || (dy == 0 && dz == 0);
+                if (half) c[dx] *= 0.5;
+                pairs += half ? 1 : 2;
                 if (lo < 0) lo = dx / 4;
                 hi = dx / 4;
             }
@@ -335,6 +341,7 @@ static void tail_direct_rows(const Geom& g, int sigma, double rcut, double eps, 
                                            (float)(c[j + 3] * (j + 3))));
             }
         }
+    return pairs;
 }
 
 static int ball_count(int sigma)
@@ -611,11 +618,22 @@ static int create_impl(lbif_handle* out, int nx, int ny, int nz, int sigma, int 
         if (!h->tail_fft) {
             std::vector<TailRow> rows;
             std::vector<float4> coef;
-            tail_direct_rows(g, sigma, F.rcut, F.eps, rows, coef);
+            const int pairs = tail_direct_rows(g, sigma, F.rcut, F.eps, rows, coef);
+            std::vector<int> off;
+            if (tail_by_pairs(g, pairs, (int)coef.size() / 2)) {
+                std::vector<int> dx, dy, dz;
+                std::vector<float4> K;
+                tail_pairs(sigma, F.rcut, F.eps, dx, dy, dz, K);
+                for (size_t k = 0; k < K.size(); ++k) off.push_back(padded_offset(g, dx[k], dy[k], dz[k]));
+                coef.swap(K);
+                rows.clear();
+                h->tail_npairs = (int)off.size();
+            }
             h->tail_nrows = (int)rows.size();
             // (never empty allocations)
             cudaError_t e = cudaMalloc((void**)&h->tail_rows, sizeof(TailRow) * (rows.size() + 1));
             if (e == cudaSuccess) e = cudaMalloc((void**)&h->tail_coef, sizeof(float4) * (coef.size() + 1));
+            if (e == cudaSuccess && !off.empty()) e = cudaMalloc((void**)&h->tail_off, sizeof(int) * off.size());
             if (e != cudaSuccess) {
                 cudaGetLastError();
                 free_ctx(h);
@@ -625,6 +643,9 @@ static int create_impl(lbif_handle* out, int nx, int ny, int nz, int sigma, int 
                                 h->stream));
             CKC(cudaMemcpyAsync(h->tail_coef, coef.data(), sizeof(float4) * coef.size(), cudaMemcpyHostToDevice,
                                 h->stream));
+            if (h->tail_off)
+                CKC(cudaMemcpyAsync(h->tail_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice,
+                                    h->stream));
             CKC(cudaStreamSynchronize(h->stream));
         }
     }

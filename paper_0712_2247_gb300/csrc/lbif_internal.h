@@ -165,6 +165,11 @@ struct TailRow {
 };
 cudaError_t launch_tail(const Params& P, const float* dn, const TailRow* rows, int nrows, const float4* coef,
                         float4* Ft, cudaStream_t s);
+// the same sum pair by pair (padded offsets and weights of the displacements of a
+// half space), and whether it is the faster one for that many pairs and chunks
+bool tail_by_pairs(const Geom& g, int pairs, int chunks);
+cudaError_t launch_tail_pairs(const Params& P, const float* dn, const int* off, const float4* K, int npairs, float4* Ft,
+                              cudaStream_t s);
 // group: edge (nodes) of the x-y block the resident CTAs sweep together (<= 0: default)
 cudaError_t launch_force(const Params& P, const Fields& f, const float4* Ft, float4* F, int group,
                          cudaStream_t s);

@@ -704,6 +704,32 @@ __global__ void __launch_bounds__(32 * TAIL_WARPS, 2) k_tail(Params P, const flo
     Ft[((long long)z * g.ny + y) * g.nx + x + warp] = make_float4(pre * t[0], pre * t[1], pre * t[2], 0.f);
 }
 
+// Shells of few pairs (a cut-off just above sigma): one node per thread, pair by
+// pair, which needs no zero coefficients, no sums across warps and two loads a pair
+// (tail_by_pairs says when).
+__global__ void __launch_bounds__(256) k_tail_pairs(Params P, const float* __restrict__ dn, const int* __restrict__ off,
+                                                    const float4* __restrict__ K, int npairs, float4* __restrict__ Ft)
+{
+    const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (idx >= P.g.N) return;
+    int x, y, z;
+    decompose(P.g, idx, x, y, z);
+    const int s = slit_of(P, z);
+    if (s < 0 || frozen(P, s)) return;
+    const float* p = dn + pidx(P.g, x, y, z);
+    float sx = 0.f, sy = 0.f, sz = 0.f;
+    for (int k = 0; k < npairs; ++k) {
+        const int o = __ldg(off + k);
+        const float d = __ldg(p + o) - __ldg(p - o);
+        const float4 c = __ldg(K + k);
+        sx = fmaf(c.x, d, sx);
+        sy = fmaf(c.y, d, sy);
+        sz = fmaf(c.z, d, sz);
+    }
+    const float pre = P.sl[s].rho0 * (1.f + __ldg(p));
+    Ft[idx] = make_float4(pre * sx, pre * sy, pre * sz, 0.f);
+}
+
 // ---------------------------------------------------------------------------
 // outputs
 // ---------------------------------------------------------------------------
@@ -1061,6 +1087,20 @@ cudaError_t launch_tail(const Params& P, const float* dn, const TailRow* rows, i
 {
     const long long nb = (long long)((P.g.nx + 3) / 4) * P.g.ny * P.g.nz;
     k_tail<<<nblocks(nb, 32), 32 * TAIL_WARPS, 0, s>>>(P, dn, rows, nrows, coef, Ft);
+    return cudaGetLastError();
+}
+
+// The rows' kernel pays per chunk of four dx (two thirds or less of it terms), the
+// pairs' per pair, and needs more nodes to fill the chip the more pairs there are.
+// Microseconds by rows / by pairs on 37 x 271 x 22 and 27 x 20 x 40: 3 pairs (3 chunks) 15.6 /
+// 7.9 and 7.7 / 6.7, 15 (9) 19.3 / 10.2 and 8.0 / 8.5, 48 (15) 22.0 / 16.6 and 8.0 / 11.9,
+// 132 (45) 37.3 / 35.8 and 11.7 / 22.4, but 115 (26) 28.4 / 31.4, 337 (81) 50.8 / 79.7.
+bool tail_by_pairs(const Geom& g, int pairs, int chunks) { return 2 * pairs <= 7 * chunks && g.N >= 1500LL * pairs; }
+
+cudaError_t launch_tail_pairs(const Params& P, const float* dn, const int* off, const float4* K, int npairs, float4* Ft,
+                              cudaStream_t s)
+{
+    k_tail_pairs<<<nblocks(P.g.N, 256), 256, 0, s>>>(P, dn, off, K, npairs, Ft);
     return cudaGetLastError();
 }
 

@@ -12,7 +12,7 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-def stack(H, nx, ny, sigma=4):
+def stack(H, nx, ny, sigma=4, rcut=2.5):
     """An Ensemble with the tail on (its constructor leaves it off)."""
     from paper_0712_2247_gb300 import lbif
 
@@ -20,7 +20,7 @@ def stack(H, nx, ny, sigma=4):
         def __init__(self):
             self._lib = lbif.load_library()
             n = len(H)
-            f = lbif.Force((ctypes.c_double * 3)(), 1, 1, 1, 0, 1, 0.2, 2.5, 0, 0)
+            f = lbif.Force((ctypes.c_double * 3)(), 1, 1, 1, 0, 1, 0.2, rcut, 0, 0)
             o = lbif.Opts(0, 3, 0.0, None, 1)
             Hc = np.asarray(H, np.int32)
             a = [np.full(n, v) for v in (0.2, 1e-6, 0.9)]
