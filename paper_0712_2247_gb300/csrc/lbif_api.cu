@@ -409,14 +409,15 @@ static int check_common(double sigma, const lbif_force& F, const lbif_opts& O, c
 // (a padded grid much larger than the nodes), and sooner where a captured graph has
 // hidden most of the launches already (ensembles). Microseconds per step without /
 // with it: 16 x 16 x 32 26.7 / 20.0, 32 x 32 x 64 at sigma 8 34.9 / 31.4, 300 x 5 x 40 31.9 /
-// 25.5, but 40 x 40 x 64 at sigma 10 43.6 / 53.0, 512 x 512 x 192 4583 / 4713, 1 x 300 x 100
-// at sigma 12 (1.1 M padded nodes) 120 / 171, 1 x 1 x 20000 (2.2 M) 71 / 132, 2 x 2 x 5000
+// 25.5, 4 x 4 x 1000 at sigma 8 (0.41 M padded nodes) 32.6 / 27.8, but 40 x 40 x 64 at
+// sigma 10 43.6 / 53.0, 512 x 512 x 192 4583 / 4713, 9 x 190 x 39 at sigma 10 (0.49 M) 73 / 95,
+// 1 x 300 x 100 at sigma 12 (1.1 M) 120 / 171, 1 x 1 x 20000 (2.2 M) 71 / 132, 2 x 2 x 5000
 // (0.6 M) 26.7 / 29.4; ensembles of 4 x 4 slits with 6,800 nodes 19.1 / 18.0, with
 // 43,500 22.8 / 24.7, 400 slits of 1 x 1 (2.0 M padded nodes) 62 / 152.
 static bool step_overlap(const Geom& g, bool batch)
 {
     const long long sms = NUM_SMS;
-    return batch ? g.N <= 128 * sms && g.P <= 1728 * sms : g.N <= 512 * sms && g.P <= 3456 * sms;
+    return batch ? g.N <= 128 * sms && g.P <= 1728 * sms : g.N <= 512 * sms && g.P <= 2688 * sms;
 }
 
 static int create_impl(lbif_handle* out, int nx, int ny, int nz, int sigma, int zper,

@@ -16,7 +16,7 @@ def kernels_us(g):
     return min(sum(g.step_profiled(20)[0].values()) for _ in range(5)) / 20 * 1e3
 
 
-@pytest.mark.parametrize("n,sigma", [((1, 1, 20000), 4), ((1, 5, 4000), 8), ((1, 300, 100), 12)])
+@pytest.mark.parametrize("n,sigma", [((1, 1, 20000), 4), ((1, 5, 4000), 8), ((1, 300, 100), 12), ((9, 190, 39), 10)])
 def test_slit(n, sigma):
     from paper_0712_2247_gb300 import lbif
 
