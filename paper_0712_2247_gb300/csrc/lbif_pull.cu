@@ -359,7 +359,7 @@ __device__ __forceinline__ void put_fields(const Params& P, const CsmIO& io, int
 // loads in flight across the two barriers of a round: 32 x 8 and 32 x 12 tiles
 // ran 7 % and 15 % slower) and marches it up a segment of z planes. Three
 // forms: two planes per round (the default, k_pull_pair below), and one plane
-// per round with the next plane's gathers issued early (k_csm) or copied by
+// per round (k_csm), with the next plane's gathers issued early or copied by
 // the tensor-memory accelerator (k_csm_tma), whose ring holds three planes.
 constexpr int CSM_TX = 32, CSM_TY = 4, CSM_THREADS = CSM_TX * CSM_TY;
 constexpr int CSM_HX = CSM_TX + 2, CSM_HN = CSM_HX * (CSM_TY + 2);  // staged nodes per plane
@@ -426,9 +426,9 @@ __device__ __forceinline__ void csm_stage(const Params& P, const CsmIO& io, cons
     }
 }
 
-// CTAs per SM the register budget of the one-plane forms is sized for, and
-// their z planes per CTA segment
-constexpr int CSM_MINB = 5;
+// CTAs per SM the register budget of the one-plane form is sized for (with and
+// without prefetching), and the z planes per CTA segment of the one-plane forms
+constexpr int CSM_MINB = 5, CSM_MINB_PLAIN = 6;
 constexpr int CSM_LZ = 16;
 
 // the stored populations of directions [I0, I1) that stream into node
@@ -547,14 +547,15 @@ __device__ __forceinline__ void csm_collide(const float* own, const float* below
     pull_gather(src, Src{own + hc}, om1s, dnr, bb, v, d79);
 }
 
-// The prefetched form: one node per thread, the population gathers of the next
-// plane issued before the current plane is staged and collided, so they are in
-// flight across both barriers (96 registers, five CTAs per SM). FP16 gathers
-// stay raw until the collision, so that the staging hides their latency.
+// One node per thread and plane. PF, the prefetched form: the population gathers of
+// the next plane issued before the current plane is staged and collided, so they
+// are in flight across both barriers (96 registers, five CTAs per SM). FP16 gathers
+// stay raw until the collision, so that the staging hides their latency. Without it
+// (80 registers, six CTAs) the form of wide slits of few planes (low_slit).
 template <typename T>
 constexpr bool F16_RAW = sizeof(T) == 2;
-template <typename T, bool IP>
-__global__ void __launch_bounds__(CSM_THREADS, CSM_MINB)
+template <typename T, bool IP, bool PF>
+__global__ void __launch_bounds__(CSM_THREADS, PF ? CSM_MINB : CSM_MINB_PLAIN)
     k_csm(Params P, const T* pin, T* pout, CsmIO io, const float4* F, int lz, int tiles_x, int tiles_y,
           int* status)
 {
@@ -588,17 +589,18 @@ __global__ void __launch_bounds__(CSM_THREADS, CSM_MINB)
     unsigned bbn;
     bool actn;
     float omn;
-    gather(zb, vn, bbn, actn, omn);
+    if constexpr (PF) gather(zb, vn, bbn, actn, omn);
     csm_stage<NT>(P, io, F, sm + csm_slot(zb - 1) * CSM_SLOT, st, zb - 1);
     csm_stage<NT>(P, io, F, sm + csm_slot(zb) * CSM_SLOT, st, zb);
     for (int z = zb; z < ze; ++z) {
+        if constexpr (!PF) gather(z, vn, bbn, actn, omn);
         float v[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) v[i] = vn[i];
         const unsigned bb = bbn;
         const bool act = actn;
         const float om = omn;
-        if (z + 1 < ze) gather(z + 1, vn, bbn, actn, omn);
+        if (PF && z + 1 < ze) gather(z + 1, vn, bbn, actn, omn);
         __syncthreads();  // the slot of plane z - 2 is free
         csm_stage<NT>(P, io, F, sm + csm_slot(z + 1) * CSM_SLOT, st, z + 1);
         __syncthreads();
@@ -1306,7 +1308,7 @@ static cudaError_t pull_any(const Params& P, const void* pin, void* pout, const 
     }
 }
 
-template <typename T, bool IP>
+template <typename T, bool IP, bool PF>
 static cudaError_t csm_tiled(const Params& P, const void* pin, void* pout, const CsmIO& io, const float4* F,
                              int* status, int lz, cudaStream_t s)
 {
@@ -1323,11 +1325,11 @@ static cudaError_t csm_tiled(const Params& P, const void* pin, void* pout, const
     if (e != cudaSuccess) return e;
     const uint64_t bit = 1ull << (dev & 63);
     if (!(configured.load() & bit)) {
-        e = cudaFuncSetAttribute(k_csm<T, IP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k_csm<T, IP, PF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         configured.fetch_or(bit);
     }
-    k_csm<T, IP><<<(unsigned)blocks, CSM_THREADS, smem, s>>>(P, (const T*)pin, (T*)pout, io, F, lz, tx, ty, status);
+    k_csm<T, IP, PF><<<(unsigned)blocks, CSM_THREADS, smem, s>>>(P, (const T*)pin, (T*)pout, io, F, lz, tx, ty, status);
     return cudaGetLastError();
 }
 
@@ -1356,6 +1358,24 @@ static cudaError_t csm_tma(const Params& P, const CUtensorMap* pmap, const void*
     return cudaGetLastError();
 }
 
+// Wide slits of few planes: most of their rounds of two planes touch a wall, where the
+// pair form steps one node after the other, and one plane a round is faster (not
+// with FP16 in two buffers, whose gathers cost that form more): prefetched, or (2)
+// plain on the widest with FP32 in two buffers. Microseconds with pairs / prefetched /
+// plain, FP32: 1000 x 1000 x 4 273 / 253 / 236, x 8 478 / 456 / 432, x 16 849 / 872 / 830,
+// 300 x 300 x 4 38.7 / 29.1 / 31.1, x 8 57 / 58 / 61; 64 x 64 x 4 14 / 21. In place: 1000 x 1000 x 8
+// FP32 480 / 420, FP16 472 / 431, x 16 861 / 830, 836 / 830. FP16 in two buffers x 8
+// 463 / 482 / 528.
+enum { LOW_NONE = 0, LOW_PREFETCHED = 1, LOW_PLAIN = 2 };
+static int low_slit(const Params& P)
+{
+    const Geom& g = P.g;
+    if (!csm_ok(g) || P.nslits > 1 || (P.storage == LBIF_STORE_F16 && !P.inplace)) return LOW_NONE;
+    const long long tiles = (long long)((g.nx + CSM_TX - 1) / CSM_TX) * ((g.ny + CSM_TY - 1) / CSM_TY);
+    if (tiles >= 4096) return g.nz > 16 ? LOW_NONE : (P.inplace ? LOW_PREFETCHED : LOW_PLAIN);
+    return tiles >= 512 && g.nz <= 6 ? LOW_PREFETCHED : LOW_NONE;
+}
+
 cudaError_t launch_csm(const Params& P, const void* pin, void* pout, const CsmIO& io, const float4* F,
                        int* status, int lz, int prefetch, cudaStream_t s, const CUtensorMap* pmap)
 {
@@ -1366,19 +1386,21 @@ cudaError_t launch_csm(const Params& P, const void* pin, void* pout, const CsmIO
         return h16 ? csm_tma<__half>(P, pmap, pin, pout, io, F, status, lz, s)
                    : csm_tma<float>(P, pmap, pin, pout, io, F, status, lz, s);
     }
-    if (prefetch != 1 || !csm_ok(g)) {
+    const int low = prefetch == 1 ? LOW_NONE : low_slit(P);
+    if ((prefetch == 1 && csm_ok(g)) || low != LOW_NONE) {
+        if (lz <= 0) lz = CSM_LZ;
         if (h16)
-            return ip ? pull_any<__half, true>(P, pin, pout, io, F, status, lz, s)
-                      : pull_any<__half, false>(P, pin, pout, io, F, status, lz, s);
-        return ip ? pull_any<float, true>(P, pin, pout, io, F, status, lz, s)
-                  : pull_any<float, false>(P, pin, pout, io, F, status, lz, s);
+            return ip ? csm_tiled<__half, true, true>(P, pin, pout, io, F, status, lz, s)
+                      : csm_tiled<__half, false, true>(P, pin, pout, io, F, status, lz, s);
+        if (ip) return csm_tiled<float, true, true>(P, pin, pout, io, F, status, lz, s);
+        return low == LOW_PLAIN ? csm_tiled<float, false, false>(P, pin, pout, io, F, status, lz, s)
+                                : csm_tiled<float, false, true>(P, pin, pout, io, F, status, lz, s);
     }
-    if (lz <= 0) lz = CSM_LZ;
     if (h16)
-        return ip ? csm_tiled<__half, true>(P, pin, pout, io, F, status, lz, s)
-                  : csm_tiled<__half, false>(P, pin, pout, io, F, status, lz, s);
-    return ip ? csm_tiled<float, true>(P, pin, pout, io, F, status, lz, s)
-              : csm_tiled<float, false>(P, pin, pout, io, F, status, lz, s);
+        return ip ? pull_any<__half, true>(P, pin, pout, io, F, status, lz, s)
+                  : pull_any<__half, false>(P, pin, pout, io, F, status, lz, s);
+    return ip ? pull_any<float, true>(P, pin, pout, io, F, status, lz, s)
+              : pull_any<float, false>(P, pin, pout, io, F, status, lz, s);
 }
 
 }  // namespace lbif
