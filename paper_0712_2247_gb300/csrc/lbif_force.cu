@@ -761,8 +761,13 @@ static void pressure4_sigma(const Params& P, const Fields& f, float* pr, cudaStr
     }
 }
 
+// Below 1024 nodes per SM the per-node kernel is the faster one: a thread's chain of
+// loads is a quarter as long, and there are enough SMs for all. Microseconds per node /
+// vectorised at sigma 4 and 12 on 64 x 64 x n: 10,000 nodes 7.7 / 8.5 and 8.4 / 11.5, 80,000
+// 7.5 / 7.6 and 7.7 / 9.8, 160,000 11.1 / 7.8 and 11.1 / 10.0, 640,000 26.0 / 14.3 and 26.8 / 15.3.
 bool launch_pressure4(const Params& P, const Fields& f, float* pr, cudaStream_t s)
 {
+    if (P.g.N < 1024LL * NUM_SMS) return false;
     switch (P.sigma) {
     case 4: pressure4_sigma<4>(P, f, pr, s); break;
     case 6: pressure4_sigma<6>(P, f, pr, s); break;

@@ -203,7 +203,7 @@ void pop_box(int storage, int* W, int* H);
 cudaError_t launch_wait_selftest(long long polls, int* status, cudaStream_t s);
 cudaError_t launch_force_soa(const Params& P, const float4* F, float* out, cudaStream_t s);
 // the pressure of every node by the vectorised kernel; false (nothing launched)
-// for a diameter without one
+// for a diameter without one and on small grids
 bool launch_pressure4(const Params& P, const Fields& f, float* pr, cudaStream_t s);
 cudaError_t launch_moments_out(const Params& P, const Fields& f, float* rho, float* u, float* p,
                                cudaStream_t s);
