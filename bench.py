@@ -112,14 +112,14 @@ def kernel_bytes(storage: int):
 
 
 # DRAM bytes per node of each step kernel (dram__bytes_read.sum + dram__bytes_write.sum of one
-# ncu capture on the 128x128x192 sigma = 12 slit, default launch shapes, divided by its nodes;
-# the pull pass: a 256x128x192 capture of k_pull_pair; the traffic scales with the nodes of a
-# launch). The ball kernel's dG writes stay in L2 at that size: read bytes only.
-TRAFFIC_B_PER_NODE = {0: {"ball_g2": 5.8, "force": 40.9, "collide_stream": 202.7},
-                      1: {"ball_g2": 5.8, "force": 40.9, "collide_stream": 126.9}}
-# the in-place pull pass (FP32, captured with the one-plane form, which moves the same lines; the FP16 in-place populations of that capture,
-# 120 MB, nearly fit in L2, so its DRAM figure does not scale and is left out)
-TRAFFIC_INPLACE = {0: {"ball_g2": 5.8, "force": 40.9, "collide_stream": 197.1}}
+# ncu capture on the 256x128x192 sigma = 12 slit, default launch shapes, divided by its nodes;
+# the traffic scales with the nodes of a launch). The ball kernel's dG writes stay in L2 at that
+# size: read bytes only.
+TRAFFIC_B_PER_NODE = {0: {"ball_g2": 5.2, "force": 44.1, "collide_stream": 203.2},
+                      1: {"ball_g2": 5.2, "force": 44.1, "collide_stream": 127.4}}
+# the same with the populations in place
+TRAFFIC_INPLACE = {0: {"ball_g2": 5.2, "force": 44.1, "collide_stream": 200.4},
+                   1: {"ball_g2": 5.2, "force": 44.1, "collide_stream": 123.5}}
 
 
 def max_over_ranks(x: float, world: int, device: str = "cuda") -> float:

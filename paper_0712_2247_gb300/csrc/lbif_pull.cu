@@ -638,11 +638,11 @@ __global__ void __launch_bounds__(CSM_THREADS, PF ? CSM_MINB : CSM_MINB_PLAIN)
 // computed once, and a round of two planes costs two barriers. Populations
 // stay scalar loads (one per node and direction), so the form has no
 // alignment condition and serves both storage layouts. Against one plane per
-// round and thread (the former default): 690 instructions per node for 1261,
+// round and thread (the former default): 705 instructions per node for 1261,
 // and at 512 x 512 x 192, sigma 12, 2.39 -> 2.19 ms FP32 (0.66 of the copy
 // bandwidth at 196 B/node), 2.54 -> 1.90 ms FP16, 2.50 -> 2.34 ms FP32 in
 // place; 256 stacked slits FP16 in place 0.68 -> 0.59 ms. It waits on load
-// latency (14 warps per SM, 37 % issue): four CTAs per SM by registers (128)
+// latency (14 warps per SM, 39 % issue): four CTAs per SM by registers (128)
 // and shared memory. Tried and slower: three CTAs with the next round's
 // gathers held in registers (2.32 ms), five CTAs at 96 registers (3.0 ms),
 // prefetching the next round's rows to L2 (2.11-2.27 ms FP32 by what it
@@ -1124,7 +1124,8 @@ __global__ void __launch_bounds__(CSM_THREADS, 4)
 // where the periodic neighbours in x and y are found by wrapping. The same code
 // forms and uses the quantities as in the marched forms (identical results).
 // 2048 slits of 4 x 4 x H: one node per thread without staging, each forming
-// its ~35 sources' quantities itself, 339 us; so 225 us.
+// its ~35 sources' quantities itself, 339 us; so 225 us (130 with the shorter
+// padded rows of later).
 // Cross-sections of up to BLOCK_A_MAX nodes run so too where the marched tiles
 // would be less than two thirds full. Microseconds in tiles / whole planes: 65 x 1 x
 // 1600 28.9 / 17.4 (25.3 without staging), 33 x 2 x 1500 28.8 / 16.5, 13 x 6 x 20000
